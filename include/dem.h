@@ -170,7 +170,8 @@ typedef struct dem_stats {
   int64_t mesh_candidates;/* particle-element candidates in the current list */
   int32_t max_list_len;   /* longest per-particle candidate list */
   int32_t status;         /* sticky device status (DEM_OK if none) */
-  int32_t launches_per_step;    /* kernels launched in a step without a list rebuild */
+  int32_t launches_per_step;    /* kernels of a step without a list rebuild (a batch of
+                                   steps adds two one-thread kernels) */
   int32_t launches_per_rebuild; /* additional kernels launched in a step that rebuilds */
   int64_t active;         /* active particles (rows 0 .. active-1); the rest await spawning */
   int64_t capacity;       /* particle rows n_cap */
@@ -181,8 +182,8 @@ typedef struct dem_scene dem_scene;
 /* Create a scene on the current CUDA device.  `stream` is a cudaStream_t (NULL:
  * the library creates its own).  Copies the host arrays to the device (the
  * particle state of Sec. 2.1 / Table 3, the mesh elements of Sec. 3.3) and
- * captures the step sequence into CUDA graphs (1 and 16 steps, for a start
- * at an even and at an odd step), which dem_step replays.
+ * captures the step sequence into CUDA graphs (a loop over batches of 1 and of
+ * 8 steps), which dem_step replays.
  * Errors: DEM_ERR_INVALID (parameters outside Table 2's requirements, n < 1,
  * non-finite input, bad element), DEM_ERR_NOMEM, DEM_ERR_CUDA. */
 int dem_scene_create(const dem_params* params, const dem_particles* particles,

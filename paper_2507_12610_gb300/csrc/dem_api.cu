@@ -16,7 +16,14 @@ using namespace dem;
 
 namespace {
 
-constexpr int kGraphSteps = 16;  // steps per replay of the long graph
+// Steps per batch of the long step graph: a loop node whose body checks for a
+// list rebuild (a conditional node), then runs this many steps.  A conditional
+// node costs about 8 us, a kernel that returns at once about 1 us, so the
+// check is made once per batch: the steps of a batch that find the lists due
+// for a rebuild return at once and are taken by the next batch.  Measured per
+// step beside the step's own kernel (8 blocks): a conditional node in every
+// step 11.1 us, batches of 1 / 4 / 8 / 16 steps 10.2 / 4.5 / 3.4 / 2.9 us.
+constexpr int kGraphSteps = 8;
 
 // Device memory of a scene: cudaMalloc, or the caller's allocator
 // (dem_scene_create_with_allocator).  Every block is released with the scene.
@@ -174,13 +181,12 @@ struct dem_scene {
   double* forces = nullptr;
   double* export_buf = nullptr;  // [13 n] state read-back staging (caller order)
   Alloc mem;
-  // step graphs (1 and kGraphSteps steps) for a start at an even / odd step:
-  // each captured step passes its kernels the pose buffers of its parity
-  cudaGraphExec_t exec1[2] = {nullptr, nullptr}, execG[2] = {nullptr, nullptr};
-  int64_t step_host = 0;  // the step the device is at once the queued work ends
-  cudaStream_t aux = nullptr;  // captures the conditional rebuild bodies
-  // branch of a captured step that computes the next step's mesh pose beside
-  // the step kernel (fork and join events)
+  // step graphs with 1 and kGraphSteps steps per batch (conditional graphs: a
+  // loop over batches, so one launch runs any number of steps; else one batch)
+  cudaGraphExec_t exec1 = nullptr, execG = nullptr;
+  cudaStream_t aux = nullptr;  // captures the bodies of the loop node
+  // captures the rebuild bodies, and the branch of a step that computes the
+  // next step's mesh pose beside the step kernels (fork and join events)
   cudaStream_t pose_stream = nullptr;
   cudaEvent_t pose_fork = nullptr, pose_join = nullptr;
   bool conditional_graphs = false;
@@ -274,88 +280,106 @@ inline void split(double a, float& hi, float& lo) {
   lo = (float)(a - (double)hi);
 }
 
-// The mesh pose of the step after `step`.  It depends on the step number
-// only, so in a capture it is a branch of its own beside the step's kernels
-// (joined before the step advances); the pose of the step itself is already
-// in its buffer (computed by the previous step, or at upload).
-cudaError_t fork_next_pose(dem_scene* s, int64_t step) {
-  if (s->static_mesh) return cudaSuccess;
-  cudaError_t e = cudaEventRecord(s->pose_fork, s->stream);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(s->pose_stream, s->pose_fork, 0);
+// The kernels of one step after the rebuild check.  The mesh pose of the next
+// step depends on the step number only: the step kernel has blocks for it, or
+// (DEM_FP64) it is a branch of its own beside the step's kernels, joined
+// before the step advances.
+cudaError_t enqueue_step(dem_scene* s, cudaStream_t st) {
+  const bool turning = !s->static_mesh;
+  const bool inside = turning && step_poses(s->p);
+  launch_spawn(st, s->ctl, s->p, s->sb, s->bb, s->mesh);
+  cudaError_t e = cudaSuccess;
+  if (turning && !inside) {
+    e = cudaEventRecord(s->pose_fork, st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s->pose_stream, s->pose_fork, 0);
+    if (e != cudaSuccess) return e;
+    launch_mesh_pose(s->pose_stream, s->ctl, s->p, s->mesh, 1);
+    e = cudaEventRecord(s->pose_join, s->pose_stream);
+    if (e != cudaSuccess) return e;
+  }
+  launch_step(st, s->ctl, s->p, s->sb, s->L, s->mesh, s->forces, inside);
+  if (turning && !inside) e = cudaStreamWaitEvent(st, s->pose_join, 0);
   if (e != cudaSuccess) return e;
-  launch_mesh_pose(s->pose_stream, s->ctl, s->p, mesh_at(s->mesh, step + 1), 1);
-  return cudaEventRecord(s->pose_join, s->pose_stream);
-}
-cudaError_t join_next_pose(dem_scene* s) {
-  if (s->static_mesh) return cudaSuccess;
-  return cudaStreamWaitEvent(s->stream, s->pose_join, 0);
-}
-
-// Enqueue one complete step on the stream (inside a capture); `step` is the
-// step number it will run at (only its parity matters).
-cudaError_t enqueue_step(dem_scene* s, int64_t step) {
-  cudaError_t e = fork_next_pose(s, step);
-  if (e != cudaSuccess) return e;
-  const MeshDev mesh = mesh_at(s->mesh, step);
-  launch_rebuild(s->stream, s->ctl, s->p, s->sb, s->L, s->bb, mesh);
-  launch_spawn(s->stream, s->ctl, s->p, s->sb, s->bb, mesh);
-  launch_step(s->stream, s->ctl, s->p, s->sb, s->L, mesh, s->forces);
-  e = join_next_pose(s);
-  if (e != cudaSuccess) return e;
-  launch_advance(s->stream, s->ctl, s->p);
+  launch_advance(st, s->ctl, s->p);
   return cudaSuccess;
 }
 
-// One step inside a stream capture, with the rebuild kernels in the body of a
-// conditional (IF) graph node whose condition a one-thread kernel sets from
-// ctl->rebuild: steps without a rebuild then launch only the step kernels.
-cudaError_t enqueue_step_conditional(dem_scene* s, int64_t step) {
-  cudaError_t e = fork_next_pose(s, step);
-  if (e != cudaSuccess) return e;
-  const MeshDev mesh = mesh_at(s->mesh, step);
+// A conditional node at the end of the capture on `st`; its body graph goes to
+// *body.
+cudaError_t add_conditional(cudaStream_t st, cudaGraphConditionalHandle h,
+                            cudaGraphConditionalNodeType type, cudaGraph_t* body) {
   cudaStreamCaptureStatus cs;
   cudaGraph_t g = nullptr;
   const cudaGraphNode_t* deps = nullptr;
   size_t nd = 0;
-  e = cudaStreamGetCaptureInfo(s->stream, &cs, nullptr, &g, nullptr, nullptr, nullptr);
-  if (e != cudaSuccess) return e;
-  cudaGraphConditionalHandle h;
-  e = cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault);
-  if (e != cudaSuccess) return e;
-  launch_decide(s->stream, s->ctl, h);
-  e = cudaStreamGetCaptureInfo(s->stream, &cs, nullptr, &g, &deps, nullptr, &nd);
+  cudaError_t e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, &deps, nullptr, &nd);
   if (e != cudaSuccess) return e;
   cudaGraphNodeParams np = {};
   np.type = cudaGraphNodeTypeConditional;
   np.conditional.handle = h;
-  np.conditional.type = cudaGraphCondTypeIf;
+  np.conditional.type = type;
   np.conditional.size = 1;
   cudaGraphNode_t node;
   e = cudaGraphAddNode(&node, g, deps, nullptr, nd, &np);
   if (e != cudaSuccess) return e;
-  cudaGraph_t body = np.conditional.phGraph_out[0];
+  *body = np.conditional.phGraph_out[0];
+  return cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1,
+                                             cudaStreamSetCaptureDependencies);
+}
+
+cudaError_t capture_graph(cudaStream_t st, cudaGraph_t* g) {
+  cudaStreamCaptureStatus cs;
+  return cudaStreamGetCaptureInfo(st, &cs, nullptr, g, nullptr, nullptr, nullptr);
+}
+
+// Inside a capture on s->aux: a batch of steps, preceded by the rebuild
+// kernels in the body of a conditional (IF) node whose condition a one-thread
+// kernel sets from ctl->rebuild.
+cudaError_t enqueue_batch(dem_scene* s, int nsteps) {
+  cudaGraph_t g = nullptr, body = nullptr;
+  cudaError_t e = capture_graph(s->aux, &g);
+  if (e != cudaSuccess) return e;
+  cudaGraphConditionalHandle h;
+  e = cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault);
+  if (e != cudaSuccess) return e;
+  launch_decide(s->aux, s->ctl, h);
+  e = add_conditional(s->aux, h, cudaGraphCondTypeIf, &body);
+  if (e != cudaSuccess) return e;
+  e = cudaStreamBeginCaptureToGraph(s->pose_stream, body, nullptr, nullptr, 0,
+                                    cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
+  launch_rebuild(s->pose_stream, s->ctl, s->p, s->sb, s->L, s->bb, s->mesh);
+  cudaGraph_t out = nullptr;
+  e = cudaStreamEndCapture(s->pose_stream, &out);
+  for (int i = 0; i < nsteps && e == cudaSuccess; ++i) e = enqueue_step(s, s->aux);
+  return e;
+}
+
+// Inside a capture on s->stream: batches of nsteps steps until ctl->left is
+// down to zero (or an error is set), as the body of a loop (WHILE) node.
+cudaError_t enqueue_loop(dem_scene* s, int nsteps) {
+  cudaGraph_t g = nullptr, body = nullptr;
+  cudaError_t e = capture_graph(s->stream, &g);
+  if (e != cudaSuccess) return e;
+  cudaGraphConditionalHandle h;
+  e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
+  if (e != cudaSuccess) return e;
+  e = add_conditional(s->stream, h, cudaGraphCondTypeWhile, &body);
+  if (e != cudaSuccess) return e;
   e = cudaStreamBeginCaptureToGraph(s->aux, body, nullptr, nullptr, 0,
                                     cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  launch_rebuild(s->aux, s->ctl, s->p, s->sb, s->L, s->bb, mesh);
-  cudaGraph_t body_out = nullptr;
-  e = cudaStreamEndCapture(s->aux, &body_out);
-  if (e != cudaSuccess) return e;
-  e = cudaStreamUpdateCaptureDependencies(s->stream, &node, nullptr, 1,
-                                          cudaStreamSetCaptureDependencies);
-  if (e != cudaSuccess) return e;
-  launch_spawn(s->stream, s->ctl, s->p, s->sb, s->bb, mesh);
-  launch_step(s->stream, s->ctl, s->p, s->sb, s->L, mesh, s->forces);
-  e = join_next_pose(s);
-  if (e != cudaSuccess) return e;
-  launch_advance(s->stream, s->ctl, s->p);
-  return cudaSuccess;
+  e = enqueue_batch(s, nsteps);
+  if (e == cudaSuccess) launch_again(s->aux, s->ctl, h);
+  cudaGraph_t out = nullptr;
+  const cudaError_t e2 = cudaStreamEndCapture(s->aux, &out);
+  return e != cudaSuccess ? e : e2;
 }
 
-// A graph of nsteps steps that starts at a step of parity `odd`.
-int build_graph(dem_scene* s, int nsteps, int odd, cudaGraphExec_t* out) {
-  // first choice: conditional rebuild bodies; fall back to the plain sequence
-  // (rebuild kernels that return at once) if the driver refuses
+// The graph of nsteps steps a batch.
+int build_graph(dem_scene* s, int nsteps, cudaGraphExec_t* out) {
+  // first choice: conditional nodes; fall back to the plain sequence (rebuild
+  // kernels that return at once) if the driver refuses.
   // DEM_GRAPH_CONDITIONAL=0 in the environment keeps every rebuild kernel a
   // plain graph node (profilers cannot see kernels of conditional graphs)
   const char* env = std::getenv("DEM_GRAPH_CONDITIONAL");
@@ -365,8 +389,13 @@ int build_graph(dem_scene* s, int nsteps, int odd, cudaGraphExec_t* out) {
     cudaGraph_t g = nullptr;
     DEM_TRY(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < nsteps && e == cudaSuccess; ++i) {
-      e = cond ? enqueue_step_conditional(s, odd + i) : enqueue_step(s, odd + i);
+    if (cond) {
+      e = enqueue_loop(s, nsteps);
+    } else {
+      for (int i = 0; i < nsteps && e == cudaSuccess; ++i) {
+        launch_rebuild(s->stream, s->ctl, s->p, s->sb, s->L, s->bb, s->mesh);
+        e = enqueue_step(s, s->stream);
+      }
     }
     const cudaError_t e2 = cudaStreamEndCapture(s->stream, &g);
     if (e == cudaSuccess && e2 == cudaSuccess) {
@@ -656,10 +685,8 @@ int upload_state(dem_scene* s, const double* x, const double* v, const double* w
 
 void destroy(dem_scene* s) {
   if (!s) return;
-  for (int b = 0; b < 2; ++b) {
-    if (s->exec1[b]) cudaGraphExecDestroy(s->exec1[b]);
-    if (s->execG[b]) cudaGraphExecDestroy(s->execG[b]);
-  }
+  if (s->exec1) cudaGraphExecDestroy(s->exec1);
+  if (s->execG) cudaGraphExecDestroy(s->execG);
   if (s->stream) cudaStreamSynchronize(s->stream);
   s->mem.release();
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
@@ -1020,15 +1047,11 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
     s->mesh.ref = M.get<D4>(s->nv);
     s->mesh.tri = M.get<int4>(s->nt);
     s->mesh.rad = M.get<double>(s->nt);
-    s->mesh.cur = M.get<D4>(4 * (size_t)s->nt);
-    s->mesh.curf = M.get<float4>(4 * (size_t)s->nt);
-    s->mesh.curl = M.get<float4>(4 * (size_t)s->nt);
-    s->mesh.plane = M.get<float4>(2 * (size_t)s->nt);
+    s->mesh.cur = M.get<D4>(8 * (size_t)s->nt);  // poses of an even and an odd step
+    s->mesh.curf = M.get<float4>(8 * (size_t)s->nt);
+    s->mesh.curl = M.get<float4>(8 * (size_t)s->nt);
+    s->mesh.plane = M.get<float4>(4 * (size_t)s->nt);
     s->mesh.nref = M.get<D4>(s->nt);
-    s->mesh.cur_odd = M.get<D4>(4 * (size_t)s->nt);
-    s->mesh.curf_odd = M.get<float4>(4 * (size_t)s->nt);
-    s->mesh.curl_odd = M.get<float4>(4 * (size_t)s->nt);
-    s->mesh.plane_odd = M.get<float4>(2 * (size_t)s->nt);
   }
   if (parts->n_materials > 0) {
     p.n_mat = parts->n_materials;
@@ -1102,19 +1125,14 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
   }
   if (rc != DEM_OK) return fail(rc);
   // poses of steps 0 and 1 (a static mesh keeps them)
-  s->step_host = 0;
-  launch_mesh_pose(s->stream, s->ctl, s->p, mesh_at(s->mesh, 0), 0);
-  launch_mesh_pose(s->stream, s->ctl, s->p, mesh_at(s->mesh, 1), 1);
+  launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 0);
+  launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 1);
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) return fail(DEM_ERR_CUDA);
-  // capture and instantiate the step graphs now (1 and kGraphSteps steps,
-  // both parities), so that no dem_step call pays for it on the host while
-  // the device waits; a failure here leaves them to be built on first use
-  for (int odd = 0; odd < 2; ++odd) {
-    if (!s->exec1[odd] && build_graph(s, 1, odd, &s->exec1[odd]) != DEM_OK)
-      s->exec1[odd] = nullptr;
-    if (!s->execG[odd] && build_graph(s, kGraphSteps, odd, &s->execG[odd]) != DEM_OK)
-      s->execG[odd] = nullptr;
-  }
+  // capture and instantiate the step graphs now, so that no dem_step call
+  // pays for it on the host while the device waits; a failure here leaves
+  // them to be built on first use
+  if (build_graph(s, 1, &s->exec1) != DEM_OK) s->exec1 = nullptr;
+  if (build_graph(s, kGraphSteps, &s->execG) != DEM_OK) s->execG = nullptr;
   cudaGetLastError();
   *out = s;
   return DEM_OK;
@@ -1123,19 +1141,29 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
 int dem_step(dem_scene* s, int64_t nsteps) {
   if (!s || nsteps < 0) return DEM_ERR_INVALID;
   if (nsteps == 0) return DEM_OK;
-  // graphs are built on first use, per parity of the starting step
-  int64_t left = nsteps;
-  while (left > 0) {
-    const int odd = (int)(s->step_host & 1);
-    const int k = left >= kGraphSteps ? kGraphSteps : 1;
-    cudaGraphExec_t* ex = k == kGraphSteps ? s->execG : s->exec1;
-    if (!ex[odd]) {
-      const int rc = build_graph(s, k, odd, &ex[odd]);
-      if (rc != DEM_OK) return rc;
-    }
-    DEM_TRY(cudaGraphLaunch(ex[odd], s->stream));
-    left -= k;
-    s->step_host += k;
+  // graphs are built on first use if creation could not; the first build says
+  // whether they loop on the device
+  const auto ready = [s](int k) {
+    cudaGraphExec_t* ex = k == 1 ? &s->exec1 : &s->execG;
+    return *ex ? (int)DEM_OK : build_graph(s, k, ex);
+  };
+  // a batch's steps beyond those left return at once (~1 us each); so do the
+  // loop's nodes (~8 us a batch): batches of one step pay for one or two steps
+  const int k = nsteps > 2 ? kGraphSteps : 1;
+  int rc = ready(k);
+  if (rc != DEM_OK) return rc;
+  launch_set_left(s->stream, s->ctl, nsteps);
+  DEM_TRY(cudaGetLastError());
+  if (s->conditional_graphs) {
+    DEM_TRY(cudaGraphLaunch(k == 1 ? s->exec1 : s->execG, s->stream));
+    return DEM_OK;
+  }
+  for (int64_t left = nsteps; left > 0;) {
+    const int m = left >= kGraphSteps ? kGraphSteps : 1;
+    rc = ready(m);
+    if (rc != DEM_OK) return rc;
+    DEM_TRY(cudaGraphLaunch(m == 1 ? s->exec1 : s->execG, s->stream));
+    left -= m;
   }
   return DEM_OK;
 }
@@ -1150,20 +1178,18 @@ int dem_step_timed(dem_scene* s, int64_t nsteps, double* phase_ms) {
     }
   int rc = DEM_OK;
   double acc[4] = {0, 0, 0, 0};
+  if (nsteps > 0) launch_set_left(s->stream, s->ctl, nsteps);
   for (int64_t k = 0; k < nsteps && rc == DEM_OK; ++k) {
     // phase by phase on one stream; the pose timed is that of the next step
-    const MeshDev mesh = mesh_at(s->mesh, s->step_host);
     cudaEventRecord(ev[0], s->stream);
-    if (!s->static_mesh)
-      launch_mesh_pose(s->stream, s->ctl, s->p, mesh_at(s->mesh, s->step_host + 1), 1);
+    if (!s->static_mesh) launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 1);
     cudaEventRecord(ev[1], s->stream);
-    launch_rebuild(s->stream, s->ctl, s->p, s->sb, s->L, s->bb, mesh);
-    launch_spawn(s->stream, s->ctl, s->p, s->sb, s->bb, mesh);
+    launch_rebuild(s->stream, s->ctl, s->p, s->sb, s->L, s->bb, s->mesh);
+    launch_spawn(s->stream, s->ctl, s->p, s->sb, s->bb, s->mesh);
     cudaEventRecord(ev[2], s->stream);
-    launch_step(s->stream, s->ctl, s->p, s->sb, s->L, mesh, s->forces);
+    launch_step(s->stream, s->ctl, s->p, s->sb, s->L, s->mesh, s->forces, false);
     cudaEventRecord(ev[3], s->stream);
     launch_advance(s->stream, s->ctl, s->p);
-    ++s->step_host;
     cudaEventRecord(ev[4], s->stream);
     rc = cuda_status(cudaEventSynchronize(ev[4]));
     for (int i = 0; i < 4 && rc == DEM_OK; ++i) {
@@ -1272,10 +1298,10 @@ int dem_get_stats(dem_scene* s, dem_stats* out) {
   out->active = c.n_active;
   out->capacity = s->n;
   const int32_t rebuild_launches = 15 + (s->nt > 0 ? 9 : 0) + (s->p.pair_res ? 1 : 0);
-  const int32_t base = (s->static_mesh ? 0 : 1) + 2 + (s->p.sp_attempts > 0 ? 1 : 0) +
-                       (s->p.pair_res ? 1 : 0);
+  const int32_t base = (s->static_mesh || step_poses(s->p) ? 0 : 1) + 2 +
+                       (s->p.sp_attempts > 0 ? 1 : 0) + (s->p.pair_res ? 1 : 0);
   if (s->conditional_graphs) {
-    out->launches_per_step = base + 1;
+    out->launches_per_step = base;
     out->launches_per_rebuild = rebuild_launches;
   } else {
     out->launches_per_step = base + rebuild_launches;
@@ -1426,9 +1452,8 @@ int dem_load(dem_scene* s, const void* buf, size_t len) {
   c.spawn_carry = carry;
   DEM_TRY(cudaMemcpy(s->ctl, &c, sizeof c, cudaMemcpyHostToDevice));
   launch_set_pose(s->stream, s->ctl, s->p);
-  s->step_host = step;
-  launch_mesh_pose(s->stream, s->ctl, s->p, mesh_at(s->mesh, step), 0);
-  launch_mesh_pose(s->stream, s->ctl, s->p, mesh_at(s->mesh, step + 1), 1);
+  launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 0);
+  launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 1);
   DEM_TRY(cudaStreamSynchronize(s->stream));
   return DEM_OK;
 }

@@ -26,6 +26,7 @@ struct Ctl {
   uint32_t disp_flag;   // set by the step kernel: some particle moved > skin/2
   uint32_t force_rebuild;
   int64_t step;         // steps completed
+  int64_t left;         // steps of the current dem_step call still to run
   int64_t rebuilds;
   double mesh_angle_ref;  // mesh rotation angle at the last rebuild
   double rot_c, rot_s;    // cos / sin of the mesh rotation angle of the current step
@@ -169,27 +170,22 @@ struct NoAux {};
 
 // Mesh elements (Sec. 3.3): triangles first, then points, segments and
 // rectangles; four vertex slots per element, unused slots repeat vertex 0.
-// The pose arrays (cur, curf, curl, plane) hold the pose of an even step, the
-// *_odd arrays that of an odd step: the pose of step n + 1 is computed while
-// step n runs (it depends on the step number only).  The host passes each
-// kernel the view of its step (mesh_at), so kernels index no buffer by the
-// step at run time.
+// The pose arrays (cur, curf, curl, plane) hold two poses, that of an even step
+// in their first nt elements and that of an odd step in the next nt: the pose
+// of step n + 1 is computed while step n runs (it depends on the step number
+// only).  Kernels read element k of the current pose at k + pose_at(...).
 struct MeshDev {
   D4* ref;           // [nv] reference vertices (x, y, z, 0)
   int4* tri;         // [nt] vertex indices, -1 for unused slots
   double* rad;       // [nt] element radius
-  D4* cur;           // [nt][4] current vertices (absolute); .w of slot 0 = radius
-  float4* curf;      // [nt][4] current vertices, shifted (float); .w of slot 0 = vertex count
-  float4* curl;      // [nt][4] low words of the shifted vertices (curf + curl = shifted
+  D4* cur;           // [2][nt][4] current vertices (absolute); .w of slot 0 = radius
+  float4* curf;      // [2][nt][4] current vertices, shifted (float); .w of slot 0 = vertex count
+  float4* curl;      // [2][nt][4] low words of the shifted vertices (curf + curl = shifted
                      // vertex to ~1e-15); .w of slots 0, 1 = radius (hi, lo)
-  float4* plane;     // [nt][2] face plane n.X = c in shifted coordinates, unit n:
+  float4* plane;     // [2][nt][2] face plane n.X = c in shifted coordinates, unit n:
                      // (n hi, c hi), (n lo, c lo); zero for points and segments
   D4* nref;          // [nt] unit normal of the face at the reference pose (zero for
                      // points, segments and degenerate faces)
-  D4* cur_odd;       // the four pose arrays above, for odd steps
-  float4* curf_odd;
-  float4* curl_odd;
-  float4* plane_odd;
   int32_t nv, nt;
 };
 
@@ -242,16 +238,16 @@ __device__ __forceinline__ void* buf_of(void* const (&a)[2], uint32_t b) {
 }
 size_t pair_result_bytes();  // bytes of one entry's DEM_FP64 pair result
 
-// The mesh with the pose arrays of step `step` (even or odd buffers).
-inline MeshDev mesh_at(const MeshDev& m, int64_t step) {
-  MeshDev r = m;
-  if (step & 1) {
-    r.cur = m.cur_odd;
-    r.curf = m.curf_odd;
-    r.curl = m.curl_odd;
-    r.plane = m.plane_odd;
-  }
-  return r;
+// First element of the pose of step `step` in the pose arrays.
+__device__ __forceinline__ uint32_t pose_at(const MeshDev& m, int64_t step) {
+  return (step & 1) ? (uint32_t)m.nt : 0u;
+}
+
+// Nothing to do for a step's kernels: an error is set, the lists must be
+// rebuilt first (the rest of a batch of captured steps then waits for the
+// next batch), or every step asked for is done.
+__device__ __forceinline__ bool step_idle(const Ctl* c) {
+  return c->status != 0u || c->rebuild != 0u || c->left <= 0;
 }
 
 __device__ __forceinline__ ListBuf list_of(const Lists& L, uint32_t b) {
@@ -275,13 +271,15 @@ __device__ __forceinline__ ListBuf list_of(const Lists& L, uint32_t b) {
 // Kernel launch helpers implemented in the .cu files.
 void launch_spawn(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, BinBuf bb,
                   MeshDev mesh);
-// The pose of step ctl->step + ahead (ahead 0 or 1) into the pose arrays of
-// `mesh` (the view of that step).
+// The pose of step ctl->step + ahead (ahead 0 or 1) into the pose arrays.
 void launch_mesh_pose(cudaStream_t st, const Ctl* ctl, const Params& p, MeshDev mesh, int ahead);
 void launch_rebuild(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
                     BinBuf bb, MeshDev mesh);
+// With `pose`, the step kernel also computes the pose of the next step (only
+// where step_poses says it can; else launch_mesh_pose does).
 void launch_step(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
-                 MeshDev mesh, double* forces);
+                 MeshDev mesh, double* forces, bool pose);
+bool step_poses(const Params& p);
 void launch_advance(cudaStream_t st, Ctl* ctl, const Params& p);
 // The current state in caller order as doubles: x[n][3], v[n][3], w[n][3],
 // q[n][4] one after another in `out` (13 n doubles, device memory).
@@ -289,8 +287,12 @@ void launch_export_state(cudaStream_t st, const Ctl* ctl, const Params& p, State
                          Lists L, int64_t n, double* out);
 // Sets ctl->rot_c / rot_s for the step in the control block.
 void launch_set_pose(cudaStream_t st, Ctl* ctl, const Params& p);
-// Sets a graph IF-condition from ctl->rebuild (inside a captured graph).
+// Sets the number of steps to run.
+void launch_set_left(cudaStream_t st, Ctl* ctl, int64_t left);
+// Sets a graph condition (inside a captured graph): whether the lists must be
+// rebuilt now; whether steps are left to run.
 void launch_decide(cudaStream_t st, const Ctl* ctl, cudaGraphConditionalHandle h);
+void launch_again(cudaStream_t st, const Ctl* ctl, cudaGraphConditionalHandle h);
 
 // Scan of a u32 array (exclusive) on the device; early-exits unless ctl->rebuild.
 void launch_scan(cudaStream_t st, const Ctl* ctl, const uint32_t* in, uint32_t* out, int64_t n,

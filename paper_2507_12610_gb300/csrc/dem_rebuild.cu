@@ -423,11 +423,12 @@ k_list_build(Ctl* ctl, Params p, BinBuf bb, Lists L, MeshDev mesh) {
     Hist* hpm_n = static_cast<Hist*>(ln.hpm);
     int ko2 = 0;
     const V3<float> q = mk(X.x, X.y, X.z);
+    const uint32_t pose = pose_at(mesh, ctl->step);
     bool tover = false;
     for (uint32_t i = a; i < b; ++i) {
       const uint32_t k = bb.tcell_tri[i];
-      const float4 A = mesh.curf[4 * k], B = mesh.curf[4 * k + 1], C = mesh.curf[4 * k + 2],
-                   D = mesh.curf[4 * k + 3];
+      const float4* v4 = mesh.curf + 4 * (size_t)(pose + k);
+      const float4 A = v4[0], B = v4[1], C = v4[2], D = v4[3];
       const V3<float> y = closest_point_element(q, mk(A.x, A.y, A.z), mk(B.x, B.y, B.z),
                                                 mk(C.x, C.y, C.z), mk(D.x, D.y, D.z), (int)A.w);
       const V3<float> d = q - y;
@@ -531,6 +532,7 @@ __global__ void k_rebuild_prep(Ctl* ctl, Params p) {
 __global__ void k_rebuild_end(Ctl* ctl, Params p, BinBuf bb, int nt) {
   if (!rebuilding(ctl)) return;
   if (nt > 0) bb.tcell_overflow[1] = 1u;  // element lists kept
+  ctl->rebuild = 0u;
   ctl->phase ^= 1u;
   ctl->lphase ^= 1u;
   ctl->rebuilds += 1;

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(32)
 k_spawn(Ctl* ctl, Params p, StateBufs sb, BinBuf bb, MeshDev mesh) {
   __shared__ double kx[kSpawnMaxAttempts], ky[kSpawnMaxAttempts], kz[kSpawnMaxAttempts],
       kr[kSpawnMaxAttempts];
-  if (ctl->status) return;
+  if (step_idle(ctl)) return;
   if (ctl->step % p.sp_every != 0) return;
   const uint32_t A = ctl->n_active;
   if (A >= (uint32_t)p.n) return;
@@ -117,6 +117,7 @@ k_spawn(Ctl* ctl, Params p, StateBufs sb, BinBuf bb, MeshDev mesh) {
   Rec* V = static_cast<Rec*>(buf_of(sb.V, ph));
   Rec* W = static_cast<Rec*>(buf_of(sb.W, ph));
   Rec* Q = static_cast<Rec*>(buf_of(sb.Q, ph));
+  const uint32_t pose = pose_at(mesh, ctl->step);
   uint64_t draws = ctl->spawn_draws;
   double carry = ctl->spawn_carry;
   uint32_t kept = 0;
@@ -162,9 +163,10 @@ k_spawn(Ctl* ctl, Params p, StateBufs sb, BinBuf bb, MeshDev mesh) {
       for (uint32_t i = bb.tcell_start[cell] + lane; i < e && !ov; i += 32) {
         const uint32_t k = bb.tcell_tri[i];
         const V3<double> q = mk(cx, cy, cz);
+        const uint32_t kp = pose + k;
         const V3<double> y = closest_point_element(
-            q, xyz(mesh.cur[4 * k]), xyz(mesh.cur[4 * k + 1]), xyz(mesh.cur[4 * k + 2]),
-            xyz(mesh.cur[4 * k + 3]), (int)mesh.curf[4 * k].w);
+            q, xyz(mesh.cur[4 * kp]), xyz(mesh.cur[4 * kp + 1]), xyz(mesh.cur[4 * kp + 2]),
+            xyz(mesh.cur[4 * kp + 3]), (int)mesh.curf[4 * kp].w);
         ov = overlaps(cx, cy, cz, r, Sphere{y.x, y.y, y.z, mesh.rad[k]});
       }
     }

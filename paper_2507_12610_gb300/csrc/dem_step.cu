@@ -27,29 +27,30 @@ namespace {
 
 // ---- mesh pose: reference vertices rotated by |Omega| t about the axis ------
 
-// One thread per element: its vertices at the pose of step ctl->step + ahead
-// (absolute in FP64; shifted as hi + lo floats), and for triangles and
-// rectangles the unit normal (the reference normal, rotated) and offset of
-// its plane, split the same way.  The rotation's cosine and sine are taken
-// once per block.
-constexpr int kPoseThreads = 128;
-
-__global__ void __launch_bounds__(kPoseThreads)
-k_mesh_pose(const Ctl* ctl, Params p, MeshDev mesh, int ahead) {
+// One thread per element: its vertices at the pose of step `step` (absolute
+// in FP64; shifted as hi + lo floats), and for triangles and rectangles the
+// unit normal (the reference normal, rotated) and offset of its plane, split
+// the same way.  The rotation's cosine and sine are taken once per block, by
+// two different warps where the block has them (each is a chain of dependent
+// FP64 operations).  `block`: which blockDim.x elements.  Not inlined: the
+// pose kernel and the step kernels run the same code, so a pose has the same
+// bits whichever computed it (inlined into the step kernel its multiply-adds
+// contract differently).
+__device__ __noinline__ void pose_block(const Params& p, const MeshDev& mesh, int64_t step,
+                                           int block) {
   __shared__ double s_cs[2];
-  if (ctl->status) return;  // the same for every thread of the block
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t step = ctl->step + ahead;
-  if (threadIdx.x == 0) {
-    // the pose of this step: the same expression, so the same bits, as
-    // k_set_pose, which keeps the one-thread step kernels free of FP64
-    // transcendentals
+  const int k = block * blockDim.x + threadIdx.x;
+  const int sin_thread = blockDim.x > 32 ? 32 : 0;
+  if ((int)threadIdx.x == 0 || (int)threadIdx.x == sin_thread) {
+    // the same expression, so the same bits, as k_set_pose, which keeps the
+    // one-thread step kernels free of FP64 transcendentals
     const double th = p.omega_norm * ((double)step * p.dt);
-    s_cs[0] = p.omega_norm > 0.0 ? cos(th) : 1.0;
-    s_cs[1] = p.omega_norm > 0.0 ? sin(th) : 0.0;
+    if (threadIdx.x == 0) s_cs[0] = p.omega_norm > 0.0 ? cos(th) : 1.0;
+    if ((int)threadIdx.x == sin_thread) s_cs[1] = p.omega_norm > 0.0 ? sin(th) : 0.0;
   }
   __syncthreads();
   if (k >= mesh.nt) return;
+  const uint32_t kp = pose_at(mesh, step) + (uint32_t)k;
   const int4 tv = mesh.tri[k];
   const int nvk = tv.w >= 0 ? 4 : (tv.z >= 0 ? 3 : (tv.y >= 0 ? 2 : 1));
   const double rad = mesh.rad[k];
@@ -69,12 +70,12 @@ k_mesh_pose(const Ctl* ctl, Params p, MeshDev mesh, int ahead) {
       const V3<double> r = pos - ctr;
       pos = ctr + (c * r + s * cross(ax, r) + (dot(ax, r) * (1.0 - c)) * ax);
     }
-    mesh.cur[4 * k + j] = make_D4(pos.x, pos.y, pos.z, j == 0 ? rad : 0.0);
+    mesh.cur[4 * kp + j] = make_D4(pos.x, pos.y, pos.z, j == 0 ? rad : 0.0);
     X[j] = pos - org;
     const float hx = (float)X[j].x, hy = (float)X[j].y, hz = (float)X[j].z;
     const float rw = j == 0 ? (float)rad : (j == 1 ? (float)(rad - (double)(float)rad) : 0.f);
-    mesh.curf[4 * k + j] = make_float4(hx, hy, hz, j == 0 ? (float)nvk : 0.f);
-    mesh.curl[4 * k + j] = make_float4((float)(X[j].x - hx), (float)(X[j].y - hy),
+    mesh.curf[4 * kp + j] = make_float4(hx, hy, hz, j == 0 ? (float)nvk : 0.f);
+    mesh.curl[4 * kp + j] = make_float4((float)(X[j].x - hx), (float)(X[j].y - hy),
                                        (float)(X[j].z - hz), rw);
   }
   // the face normal: the reference one, rotated like the vertices
@@ -87,8 +88,16 @@ k_mesh_pose(const Ctl* ctl, Params p, MeshDev mesh, int ahead) {
     pl = make_float4((float)(nrm.x - ph.x), (float)(nrm.y - ph.y), (float)(nrm.z - ph.z),
                      (float)(off - ph.w));
   }
-  mesh.plane[2 * k] = ph;
-  mesh.plane[2 * k + 1] = pl;
+  mesh.plane[2 * kp] = ph;
+  mesh.plane[2 * kp + 1] = pl;
+}
+
+constexpr int kPoseThreads = 64;
+
+__global__ void __launch_bounds__(kPoseThreads)
+k_mesh_pose(const Ctl* ctl, Params p, MeshDev mesh, int ahead) {
+  if (ctl->status) return;  // the same for every thread of the block
+  pose_block(p, mesh, ctl->step + ahead, blockIdx.x);
 }
 
 // Rotation of the mesh at the control block's step (after a host upload); the
@@ -105,12 +114,21 @@ __global__ void k_decide(const Ctl* ctl, cudaGraphConditionalHandle h) {
   cudaGraphSetConditional(h, (ctl->rebuild != 0u && ctl->status == 0u) ? 1u : 0u);
 }
 
+// ---- graph condition: another batch of steps, or all done -------------------
+
+__global__ void k_again(const Ctl* ctl, cudaGraphConditionalHandle h) {
+  cudaGraphSetConditional(h, (ctl->left > 0 && ctl->status == 0u) ? 1u : 0u);
+}
+
+__global__ void k_set_left(Ctl* ctl, int64_t left) { ctl->left = left; }
+
 // ---- end of step: flip buffers, count, decide the next rebuild -------------
 
 __global__ void k_advance(Ctl* ctl, Params p) {
-  if (ctl->status) return;
+  if (step_idle(ctl)) return;
   ctl->phase ^= 1u;
   ctl->step += 1;
+  ctl->left -= 1;
   ctl->pair_contacts_last = ctl->pair_contacts;
   ctl->mesh_contacts_last = ctl->mesh_contacts;
   ctl->pair_contacts = 0;
@@ -246,6 +264,11 @@ __device__ __forceinline__ bool mesh_gap(const MeshDev& mesh, uint32_t kt, int f
 }
 
 struct MixedPolicy {
+  // mesh pose of the next step, by extra blocks of the step kernel
+  static __device__ __forceinline__ void pose(const Params& p, const MeshDev& mesh, int64_t step,
+                                              int block) {
+    pose_block(p, mesh, step, block);
+  }
   static constexpr int kMinBlocks = DEM_MIXED_MIN_BLOCKS;  // resident blocks per SM
   using Rec = F8;
   using Hist = HistM;
@@ -383,12 +406,12 @@ struct MixedPolicy {
   // torque on the particle to c6.
   static __device__ __forceinline__ bool mesh_contact(const Params& p, const MeshDev& mesh,
                                                       const ListBuf& lb, int t, int m,
-                                                      const F8& Pt, const F8& Vt, const F8& Wt,
-                                                      uint32_t stamp_now, uint32_t stamp_new,
-                                                      float c6[6]) {
+                                                      uint32_t pose, const F8& Pt, const F8& Vt,
+                                                      const F8& Wt, uint32_t stamp_now,
+                                                      uint32_t stamp_new, float c6[6]) {
     const int n = p.n;
     const float Rt = Pt.hi.w + Pt.lo.w;
-    const uint32_t kt = lb.tric[(size_t)m * n + t];
+    const uint32_t kt = pose + lb.tric[(size_t)m * n + t];
     const V3<float> qf = sum3(Pt);
     const float4 Af = mesh.curf[4 * kt], Bf = mesh.curf[4 * kt + 1],
                  Cf = mesh.curf[4 * kt + 2], Df = mesh.curf[4 * kt + 3];
@@ -447,8 +470,8 @@ struct MixedPolicy {
   // and integration of particle slot t.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
-                                                const MeshDev& mesh, int t, uint32_t ntc_u,
-                                                bool with_mesh, const F8& Pt, const F8& Vt,
+                                                const MeshDev& mesh, uint32_t pose, int t,
+                                                uint32_t ntc_u, bool with_mesh, const F8& Pt, const F8& Vt,
                                                 const F8& Wt, Acc& sums, uint32_t stamp_now,
                                                 uint32_t stamp_new, double* forces,
                                                 uint32_t& nmesh, bool& disp, bool& bad) {
@@ -468,7 +491,7 @@ struct MixedPolicy {
     Acc3& T = sums.T;
     for (int m = 0; m < ntc; ++m) {
       float c6[6];
-      if (!mesh_contact(p, mesh, lb, t, m, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
+      if (!mesh_contact(p, mesh, lb, t, m, pose, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
       sums.add(c6);
       ++nmesh;
     }
@@ -553,6 +576,10 @@ struct MixedPolicy {
 #endif
 
 struct Mixed64Policy {
+  static __device__ __forceinline__ void pose(const Params& p, const MeshDev& mesh, int64_t step,
+                                              int block) {
+    pose_block(p, mesh, step, block);
+  }
   static constexpr int kMinBlocks = DEM_MIXED64_MIN_BLOCKS;
   using Rec = D4;
   using Hist = HistM;
@@ -644,15 +671,16 @@ struct Mixed64Policy {
   // overlap in FP64 (an element is large next to the overlap), the law in FP32.
   static __device__ __forceinline__ bool mesh_contact(const Params& p, const MeshDev& mesh,
                                                       const ListBuf& lb, int t, int m,
-                                                      const D4& Pt, const D4& Vt, const D4& Wt,
-                                                      uint32_t stamp_now, uint32_t stamp_new,
-                                                      float c6[6]) {
+                                                      uint32_t pose, const D4& Pt, const D4& Vt,
+                                                      const D4& Wt, uint32_t stamp_now,
+                                                      uint32_t stamp_new, float c6[6]) {
     const int n = p.n;
     const uint32_t kt = lb.tric[(size_t)m * n + t];
     const V3<double> x = xyz(Pt);
-    const D4 A = mesh.cur[4 * kt], B = mesh.cur[4 * kt + 1], C = mesh.cur[4 * kt + 2],
-             D = mesh.cur[4 * kt + 3];
-    const int nvk = (int)mesh.curf[4 * kt].w;
+    const uint32_t kp = pose + kt;
+    const D4 A = mesh.cur[4 * kp], B = mesh.cur[4 * kp + 1], C = mesh.cur[4 * kp + 2],
+             D = mesh.cur[4 * kp + 3];
+    const int nvk = (int)mesh.curf[4 * kp].w;
     const V3<double> pc = closest_point_element(x, xyz(A), xyz(B), xyz(C), xyz(D), nvk);
     const V3<double> d = x - pc;
     const double dist = sqrt(dot(d, d));
@@ -705,8 +733,8 @@ struct Mixed64Policy {
   // to the FP64 velocity, spin and orientation; positions advance in FP64.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
-                                                const MeshDev& mesh, int t, uint32_t ntc_u,
-                                                bool with_mesh, const D4& Pt, const D4& Vt,
+                                                const MeshDev& mesh, uint32_t pose, int t,
+                                                uint32_t ntc_u, bool with_mesh, const D4& Pt, const D4& Vt,
                                                 const D4& Wt, Acc& sums, uint32_t stamp_now,
                                                 uint32_t stamp_new, double* forces,
                                                 uint32_t& nmesh, bool& disp, bool& bad) {
@@ -723,7 +751,7 @@ struct Mixed64Policy {
     }
     for (int m = 0; m < ntc; ++m) {
       float c6[6];
-      if (!mesh_contact(p, mesh, lb, t, m, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
+      if (!mesh_contact(p, mesh, lb, t, m, pose, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
       sums.add(c6);
       ++nmesh;
     }
@@ -790,20 +818,37 @@ void launch_mesh_pose(cudaStream_t st, const Ctl* ctl, const Params& p, MeshDev 
 }
 
 void launch_step(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
-                 MeshDev mesh, double* forces) {
+                 MeshDev mesh, double* forces, bool pose) {
   if (p.mixed && p.pair_res)  // one evaluation per pair
     launch_step_pairs<MixedPolicy, MixedPolicy::kMinBlocks, MixedPolicy::kMinBlocks>(
         st, ctl, p, sb, L, mesh, forces);
   else if (p.mixed)
-    launch_step_warp<MixedPolicy>(st, ctl, p, sb, L, mesh, forces);
+    launch_step_warp<MixedPolicy>(st, ctl, p, sb, L, mesh, forces, pose);
   else if (p.mixed64)
-    launch_step_warp<Mixed64Policy>(st, ctl, p, sb, L, mesh, forces);
+    launch_step_warp<Mixed64Policy>(st, ctl, p, sb, L, mesh, forces, pose);
   else
     launch_step_fp64(st, ctl, p, sb, L, mesh, forces);
 }
 
+// Where the step kernel computes the next step's mesh pose in extra blocks of
+// its own instead of a graph branch beside it.  The branch's fork and join cost
+// a step about 4 us; the call costs the kernel 20 bytes of spilled registers,
+// 5 % of a step at n = 1,000,000 (288 us against 274 us with the branch), so
+// the two meet where a step takes about 80 us.
+bool step_poses(const Params& p) {
+  return p.n <= 200000 && ((p.mixed && !p.pair_res) || p.mixed64);
+}
+
 void launch_set_pose(cudaStream_t st, Ctl* ctl, const Params& p) {
   k_set_pose<<<1, 1, 0, st>>>(ctl, p);
+}
+
+void launch_set_left(cudaStream_t st, Ctl* ctl, int64_t left) {
+  k_set_left<<<1, 1, 0, st>>>(ctl, left);
+}
+
+void launch_again(cudaStream_t st, const Ctl* ctl, cudaGraphConditionalHandle h) {
+  k_again<<<1, 1, 0, st>>>(ctl, h);
 }
 
 void launch_decide(cudaStream_t st, const Ctl* ctl, cudaGraphConditionalHandle h) {

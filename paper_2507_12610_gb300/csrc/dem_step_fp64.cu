@@ -26,6 +26,8 @@ namespace {
 #endif
 
 struct Fp64Policy {
+  // (the pose is a kernel of its own: dem_step.cu)
+  static __device__ __forceinline__ void pose(const Params&, const MeshDev&, int64_t, int) {}
   static constexpr int kMinBlocks = DEM_FP64_MIN_BLOCKS;  // resident blocks per SM
   using Rec = D4;
   using Hist = HistD;
@@ -143,15 +145,16 @@ struct Fp64Policy {
   // the force and torque on the particle to c6.
   static __device__ __forceinline__ bool mesh_contact(const Params& p, const MeshDev& mesh,
                                                       const ListBuf& lb, int t, int m,
-                                                      const D4& Pt, const D4& Vt, const D4& Wt,
-                                                      uint32_t stamp_now, uint32_t stamp_new,
-                                                      double c6[6]) {
+                                                      uint32_t pose, const D4& Pt, const D4& Vt,
+                                                      const D4& Wt, uint32_t stamp_now,
+                                                      uint32_t stamp_new, double c6[6]) {
     const int n = p.n;
     const uint32_t kt = lb.tric[(size_t)m * n + t];
     const V3<double> x = xyz(Pt);
-    const D4 A = mesh.cur[4 * kt], B = mesh.cur[4 * kt + 1], C = mesh.cur[4 * kt + 2],
-             D = mesh.cur[4 * kt + 3];
-    const int nvk = (int)mesh.curf[4 * kt].w;
+    const uint32_t kp = pose + kt;
+    const D4 A = mesh.cur[4 * kp], B = mesh.cur[4 * kp + 1], C = mesh.cur[4 * kp + 2],
+             D = mesh.cur[4 * kp + 3];
+    const int nvk = (int)mesh.curf[4 * kp].w;
     const V3<double> pc = closest_point_element(x, xyz(A), xyz(B), xyz(C), xyz(D), nvk);
     const V3<double> d = x - pc;
     const double dist = sqrt(dot(d, d));
@@ -197,8 +200,8 @@ struct Fp64Policy {
   // and integration of particle slot t.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
-                                                const MeshDev& mesh, int t, uint32_t ntc_u,
-                                                bool with_mesh, const D4& Pt, const D4& Vt,
+                                                const MeshDev& mesh, uint32_t pose, int t,
+                                                uint32_t ntc_u, bool with_mesh, const D4& Pt, const D4& Vt,
                                                 const D4& Wt, Acc& sums, uint32_t stamp_now,
                                                 uint32_t stamp_new, double* forces,
                                                 uint32_t& nmesh, bool& disp, bool& bad) {
@@ -218,7 +221,7 @@ struct Fp64Policy {
     // particle-element contacts
     for (int m = 0; m < ntc; ++m) {
       double c6[6];
-      if (!mesh_contact(p, mesh, lb, t, m, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
+      if (!mesh_contact(p, mesh, lb, t, m, pose, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
       sums.add(c6);
       ++nmesh;
     }
@@ -281,7 +284,7 @@ void launch_step_fp64(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, 
     launch_step_pairs<Fp64Policy, Fp64Policy::kMinBlocks, Fp64Policy::kMinBlocks>(
         st, ctl, p, sb, L, mesh, forces);
   else  // both sides evaluate each pair (one kernel)
-    launch_step_warp<Fp64Policy>(st, ctl, p, sb, L, mesh, forces);
+    launch_step_warp<Fp64Policy>(st, ctl, p, sb, L, mesh, forces, false);
 }
 
 size_t pair_result_bytes() { return sizeof(PairOut<double>); }

@@ -87,7 +87,7 @@ k_pairs(Ctl* ctl, Params p, StateBufs sb, Lists L, PairOut<typename Pol::T>* res
   __shared__ uint8_t qlane_s[kPairWarps][kQueueMax];
   __shared__ uint8_t qk_s[kPairWarps][kQueueMax];
   __shared__ uint8_t nlow_s[kPairWarps][32];
-  if (ctl->status) return;
+  if (step_idle(ctl)) return;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   uint32_t* seg = seg_s[wib];
@@ -182,7 +182,7 @@ k_gather(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh,
          const PairOut<typename Pol::T>* res, unsigned long long* touch, double* forces) {
   using Rec = typename Pol::Rec;
   using CT = typename Pol::T;
-  if (ctl->status) return;
+  if (step_idle(ctl)) return;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = t < p.n;
   const uint32_t ph = ctl->phase & 1u, lph = ctl->lphase & 1u;
@@ -210,7 +210,7 @@ k_gather(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh,
       get_out(res + e, !lower, c6);
       acc.add(c6);
     }
-    Pol::finish(p, sb, ph, lb, mesh, t, (meta >> 16) & 0xffu, true, P[t], V[t], W[t], acc,
+    Pol::finish(p, sb, ph, lb, mesh, pose_at(mesh, ctl->step), t, (meta >> 16) & 0xffu, true, P[t], V[t], W[t], acc,
                 stamp_now, stamp_new, forces, nmesh, disp, bad);
   }
   count_and_flag(ctl, 0u, nmesh, disp, bad);

@@ -59,19 +59,24 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
   return v;
 }
 
-template <typename Pol, int Warps>
+template <typename Pol, int Warps, bool Pose>
 __global__ void __launch_bounds__(32 * Warps, (Pol::kMinBlocks * 4 / Warps > 0 ? Pol::kMinBlocks * 4 / Warps : 1))
-k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* forces) {
+k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* forces, int npose) {
   using Rec = typename Pol::Rec;
   using Hist = typename Pol::Hist;
   using CT = typename Pol::T;
   __shared__ WarpScratch<CT> smem[Warps];
-  if (ctl->status) return;
+  if (step_idle(ctl)) return;
+  // the first npose blocks compute the mesh pose of the next step
+  if (Pose && (int)blockIdx.x < npose) {
+    Pol::pose(p, mesh, ctl->step + 1, blockIdx.x);
+    return;
+  }
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   WarpScratch<CT>& S = smem[wib];
   const int n = p.n;
-  const int w0 = (blockIdx.x * Warps + wib) * 32;
+  const int w0 = (((int)blockIdx.x - (Pose ? npose : 0)) * Warps + wib) * 32;
   const int t = w0 + lane;
   const bool valid = t < n;
   const uint32_t ph = ctl->phase & 1u, lph = ctl->lphase & 1u;
@@ -220,8 +225,8 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
         for (int step = 16; step > 0; step >>= 1)
           if (S.seg[lo + step] <= c) lo += step;
         const int tl = lo;
-        hit = Pol::mesh_contact(p, mesh, lb, w0 + tl, (int)(c - S.seg[tl]), P[w0 + tl],
-                                V[w0 + tl], W[w0 + tl], stamp_now, stamp_new, c6);
+        hit = Pol::mesh_contact(p, mesh, lb, w0 + tl, (int)(c - S.seg[tl]),
+                                pose_at(mesh, ctl->step), P[w0 + tl], V[w0 + tl], W[w0 + tl], stamp_now, stamp_new, c6);
         if (hit) ++nmesh;
       }
       const unsigned hm = __ballot_sync(full, hit);
@@ -239,21 +244,31 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
   // C: integration of the lane's own particle
   bool disp = false, bad = false;
   if (valid)
-    Pol::finish(p, sb, ph, lb, mesh, t, (meta >> 16) & 0xffu, false, P[t], V[t],
+    Pol::finish(p, sb, ph, lb, mesh, 0u, t, (meta >> 16) & 0xffu, false, P[t], V[t],
                 W[t], acc, stamp_now, stamp_new, forces, nmesh, disp, bad);
 
   count_and_flag(ctl, npair, nmesh, disp, bad);
 }
 
+template <typename Pol, int Warps>
+void launch_step_warp_as(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
+                         MeshDev mesh, double* forces, bool pose) {
+  constexpr int kThreads = 32 * Warps;
+  const int npose = pose ? (mesh.nt + kThreads - 1) / kThreads : 0;
+  const unsigned nb = (unsigned)((p.n + kThreads - 1) / kThreads + npose);
+  if (pose)
+    k_step_warp<Pol, Warps, true><<<nb, kThreads, 0, st>>>(ctl, p, sb, L, mesh, forces, npose);
+  else
+    k_step_warp<Pol, Warps, false><<<nb, kThreads, 0, st>>>(ctl, p, sb, L, mesh, forces, 0);
+}
+
 template <typename Pol>
 void launch_step_warp(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
-                      MeshDev mesh, double* forces) {
+                      MeshDev mesh, double* forces, bool pose) {
   if (p.step_warps == 8)
-    k_step_warp<Pol, 8><<<(unsigned)((p.n + 255) / 256), 256, 0, st>>>(ctl, p, sb, L, mesh,
-                                                                        forces);
+    launch_step_warp_as<Pol, 8>(st, ctl, p, sb, L, mesh, forces, pose);
   else
-    k_step_warp<Pol, 4><<<(unsigned)((p.n + 127) / 128), 128, 0, st>>>(ctl, p, sb, L, mesh,
-                                                                        forces);
+    launch_step_warp_as<Pol, 4>(st, ctl, p, sb, L, mesh, forces, pose);
 }
 
 }  // namespace dem
