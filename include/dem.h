@@ -112,8 +112,9 @@ typedef struct dem_params {
   int32_t spawn_every;      /* steps between spawn events; <= 0 selects 1 */
   uint64_t spawn_seed;
   int32_t step_warps;       /* warps per block of the contact/integration kernel:
-                               4 or 8; <= 0 selects 4 (a tuning knob, results do not
-                               depend on it) */
+                               4 or 8; <= 0 selects 4 (a tuning knob for scenes of
+                               more than 80,000 particles, results do not depend
+                               on it) */
   int32_t reserved;
 } dem_params;
 

@@ -75,15 +75,9 @@ bool fp64_two_sided() {
   return env && env[0] == '1';
 }
 
-#ifndef DEM_MIXED_PAIRS
-#define DEM_MIXED_PAIRS 0
-#endif
 // Whether the step evaluates each pair once (pair kernel + gather kernel)
 // rather than from both sides in one kernel.
-bool one_eval_per_pair(const Params& p) {
-  if (p.mixed64) return false;
-  return p.mixed ? DEM_MIXED_PAIRS != 0 : !fp64_two_sided();
-}
+bool one_eval_per_pair(const Params& p) { return !p.hist32 && !fp64_two_sided(); }
 
 bool finite_all(const double* a, int64_t n) {
   for (int64_t i = 0; i < n; ++i)

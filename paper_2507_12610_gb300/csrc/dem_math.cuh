@@ -97,7 +97,6 @@ __device__ __forceinline__ void kahan(float& h, float& l, float b) {
 // Compensated accumulator of a 3-vector (order fixed by the caller).
 struct Acc3 {
   float hx, hy, hz, lx, ly, lz;
-  __device__ __forceinline__ void zero() { hx = hy = hz = lx = ly = lz = 0.f; }
   __device__ __forceinline__ void add(V3<float> v) {
     kahan(hx, lx, v.x);
     kahan(hy, ly, v.y);

@@ -18,7 +18,6 @@
 #include "dem_law.cuh"
 #include "dem_math.cuh"
 #include "dem_step_common.cuh"
-#include "dem_step_pairs.cuh"
 #include "dem_step_warp.cuh"
 
 namespace dem {
@@ -278,10 +277,6 @@ struct MixedPolicy {
 
   struct Acc {
     Acc3 F, T;
-    __device__ __forceinline__ void zero() {
-      F.zero();
-      T.zero();
-    }
     __device__ __forceinline__ void add(const float* c) {
       F.add(mk(c[0], c[1], c[2]));
       T.add(mk(c[3], c[4], c[5]));
@@ -470,12 +465,9 @@ struct MixedPolicy {
   // and integration of particle slot t.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
-                                                const MeshDev& mesh, uint32_t pose, int t,
-                                                uint32_t ntc_u, bool with_mesh, const F8& Pt, const F8& Vt,
-                                                const F8& Wt, Acc& sums, uint32_t stamp_now,
-                                                uint32_t stamp_new, double* forces,
-                                                uint32_t& nmesh, bool& disp, bool& bad) {
-    const int ntc = with_mesh ? (int)ntc_u : 0;
+                                                int t, const F8& Pt, const F8& Vt,
+                                                const F8& Wt, const Acc& sums, double* forces,
+                                                bool& disp, bool& bad) {
     const F8* Q = static_cast<const F8*>(buf_of(sb.Q, ph));
     const float Rt = Pt.hi.w + Pt.lo.w;
     if (Rt == 0.f) {  // inactive (awaiting spawning): carried over unchanged
@@ -487,14 +479,8 @@ struct MixedPolicy {
         for (int c = 0; c < 6; ++c) forces[6 * (size_t)t + c] = 0.0;
       return;
     }
-    Acc3& F = sums.F;
-    Acc3& T = sums.T;
-    for (int m = 0; m < ntc; ++m) {
-      float c6[6];
-      if (!mesh_contact(p, mesh, lb, t, m, pose, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
-      sums.add(c6);
-      ++nmesh;
-    }
+    const Acc3& F = sums.F;
+    const Acc3& T = sums.T;
     // semi-implicit Euler + SPIRAL with compensated (hi, lo) state
     const float mass = Vt.hi.w;
     const float R = Rt;
@@ -733,12 +719,9 @@ struct Mixed64Policy {
   // to the FP64 velocity, spin and orientation; positions advance in FP64.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
-                                                const MeshDev& mesh, uint32_t pose, int t,
-                                                uint32_t ntc_u, bool with_mesh, const D4& Pt, const D4& Vt,
-                                                const D4& Wt, Acc& sums, uint32_t stamp_now,
-                                                uint32_t stamp_new, double* forces,
-                                                uint32_t& nmesh, bool& disp, bool& bad) {
-    const int ntc = with_mesh ? (int)ntc_u : 0;
+                                                int t, const D4& Pt, const D4& Vt,
+                                                const D4& Wt, const Acc& sums, double* forces,
+                                                bool& disp, bool& bad) {
     const D4* Q = static_cast<const D4*>(buf_of(sb.Q, ph));
     if (Pt.w == 0.0) {  // inactive (awaiting spawning): carried over unchanged
       static_cast<D4*>(buf_of(sb.P, ph ^ 1u))[t] = Pt;
@@ -748,12 +731,6 @@ struct Mixed64Policy {
       if (p.record_forces)
         for (int c = 0; c < 6; ++c) forces[6 * (size_t)t + c] = 0.0;
       return;
-    }
-    for (int m = 0; m < ntc; ++m) {
-      float c6[6];
-      if (!mesh_contact(p, mesh, lb, t, m, pose, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
-      sums.add(c6);
-      ++nmesh;
     }
     const Acc3& F = sums.F;
     const Acc3& T = sums.T;
@@ -819,10 +796,7 @@ void launch_mesh_pose(cudaStream_t st, const Ctl* ctl, const Params& p, MeshDev 
 
 void launch_step(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
                  MeshDev mesh, double* forces, bool pose) {
-  if (p.mixed && p.pair_res)  // one evaluation per pair
-    launch_step_pairs<MixedPolicy, MixedPolicy::kMinBlocks, MixedPolicy::kMinBlocks>(
-        st, ctl, p, sb, L, mesh, forces);
-  else if (p.mixed)
+  if (p.mixed)
     launch_step_warp<MixedPolicy>(st, ctl, p, sb, L, mesh, forces, pose);
   else if (p.mixed64)
     launch_step_warp<Mixed64Policy>(st, ctl, p, sb, L, mesh, forces, pose);
@@ -836,7 +810,7 @@ void launch_step(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists
 // 5 % of a step at n = 1,000,000 (288 us against 274 us with the branch), so
 // the two meet where a step takes about 80 us.
 bool step_poses(const Params& p) {
-  return p.n <= 200000 && ((p.mixed && !p.pair_res) || p.mixed64);
+  return p.n <= 200000 && p.hist32;
 }
 
 void launch_set_pose(cudaStream_t st, Ctl* ctl, const Params& p) {

@@ -200,12 +200,9 @@ struct Fp64Policy {
   // and integration of particle slot t.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
-                                                const MeshDev& mesh, uint32_t pose, int t,
-                                                uint32_t ntc_u, bool with_mesh, const D4& Pt, const D4& Vt,
-                                                const D4& Wt, Acc& sums, uint32_t stamp_now,
-                                                uint32_t stamp_new, double* forces,
-                                                uint32_t& nmesh, bool& disp, bool& bad) {
-    const int ntc = with_mesh ? (int)ntc_u : 0;
+                                                int t, const D4& Pt, const D4& Vt,
+                                                const D4& Wt, const Acc& sums, double* forces,
+                                                bool& disp, bool& bad) {
     const D4* Q = static_cast<const D4*>(buf_of(sb.Q, ph));
     if (Pt.w == 0.0) {  // inactive (awaiting spawning): carried over unchanged
       static_cast<D4*>(buf_of(sb.P, ph ^ 1u))[t] = Pt;
@@ -216,15 +213,8 @@ struct Fp64Policy {
         for (int c = 0; c < 6; ++c) forces[6 * (size_t)t + c] = 0.0;
       return;
     }
-    V3<double>& F = sums.F;
-    V3<double>& T = sums.T;
-    // particle-element contacts
-    for (int m = 0; m < ntc; ++m) {
-      double c6[6];
-      if (!mesh_contact(p, mesh, lb, t, m, pose, Pt, Vt, Wt, stamp_now, stamp_new, c6)) continue;
-      sums.add(c6);
-      ++nmesh;
-    }
+    const V3<double>& F = sums.F;
+    const V3<double>& T = sums.T;
     // semi-implicit Euler + SPIRAL (Sec. 2.3)
     const double R = Pt.w, mass = Vt.w;  // I = 2/5 m R^2
     const double ci = 9.0 * p.eta / (2.0 * p.rho * R * R);
@@ -281,8 +271,7 @@ struct Fp64Policy {
 void launch_step_fp64(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
                       MeshDev mesh, double* forces) {
   if (p.pair_res)  // one evaluation per pair: the FP64 pipe bounds this step
-    launch_step_pairs<Fp64Policy, Fp64Policy::kMinBlocks, Fp64Policy::kMinBlocks>(
-        st, ctl, p, sb, L, mesh, forces);
+    launch_step_pairs<Fp64Policy>(st, ctl, p, sb, L, mesh, forces);
   else  // both sides evaluate each pair (one kernel)
     launch_step_warp<Fp64Policy>(st, ctl, p, sb, L, mesh, forces, false);
 }

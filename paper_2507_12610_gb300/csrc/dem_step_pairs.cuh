@@ -34,20 +34,6 @@ template <>
 struct PairOut<double> {  // 80 bytes
   double f[3], ti[3], tj[3], pad;
 };
-template <>
-struct __align__(16) PairOut<float> {  // 48 bytes
-  float f[3], ti[3], tj[3], pad[3];
-};
-
-__device__ __forceinline__ void put_out(PairOut<float>* r, const LawOut<float>& o) {
-  PairOut<float> a;
-  a.f[0] = o.f.x; a.f[1] = o.f.y; a.f[2] = o.f.z;
-  a.ti[0] = o.ti.x; a.ti[1] = o.ti.y; a.ti[2] = o.ti.z;
-  a.tj[0] = o.tj.x; a.tj[1] = o.tj.y; a.tj[2] = o.tj.z;
-  a.pad[0] = a.pad[1] = a.pad[2] = 0.f;
-  *r = a;
-}
-
 __device__ __forceinline__ void put_out(PairOut<double>* r, const LawOut<double>& o) {
   PairOut<double> a;
   a.f[0] = o.f.x; a.f[1] = o.f.y; a.f[2] = o.f.z;
@@ -68,25 +54,23 @@ __device__ __forceinline__ void get_out(const PairOut<T>* r, bool on_i, T c6[6])
   c6[3] = t[0]; c6[4] = t[1]; c6[5] = t[2];
 }
 
-constexpr int kPairWarps = 4;
-
 // Phases A and B of the warp kernel (dem_step_warp.cuh) over the warp's
 // upper entries only: a cheap overlap pre-test queues the candidates, then
 // the law runs for 32 queued pairs at a time.
-template <typename Pol, int MinBlocks>
-__global__ void __launch_bounds__(32 * kPairWarps, MinBlocks)
+template <typename Pol, int Warps, int PPW>
+__global__ void __launch_bounds__(32 * Warps, scaled_blocks(Pol::kMinBlocks, Warps))
 k_pairs(Ctl* ctl, Params p, StateBufs sb, Lists L, PairOut<typename Pol::T>* res,
         unsigned long long* touch) {
   using Rec = typename Pol::Rec;
   using Hist = typename Pol::Hist;
   using CT = typename Pol::T;
-  __shared__ uint32_t seg_s[kPairWarps][33];
-  __shared__ uint32_t off_s[kPairWarps][32];
-  __shared__ uint32_t qent_s[kPairWarps][kQueueMax];
-  __shared__ uint32_t qslot_s[kPairWarps][kQueueMax];
-  __shared__ uint8_t qlane_s[kPairWarps][kQueueMax];
-  __shared__ uint8_t qk_s[kPairWarps][kQueueMax];
-  __shared__ uint8_t nlow_s[kPairWarps][32];
+  __shared__ uint32_t seg_s[Warps][33];
+  __shared__ uint32_t off_s[Warps][32];
+  __shared__ uint32_t qent_s[Warps][kQueueMax];
+  __shared__ uint32_t qslot_s[Warps][kQueueMax];
+  __shared__ uint8_t qlane_s[Warps][kQueueMax];
+  __shared__ uint8_t qk_s[Warps][kQueueMax];
+  __shared__ uint8_t nlow_s[Warps][32];
   if (step_idle(ctl)) return;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -98,9 +82,9 @@ k_pairs(Ctl* ctl, Params p, StateBufs sb, Lists L, PairOut<typename Pol::T>* res
   uint8_t* qk = qk_s[wib];
   uint8_t* nlw = nlow_s[wib];
   const int n = p.n;
-  const int w0 = (blockIdx.x * kPairWarps + wib) * 32;
+  const int w0 = (blockIdx.x * Warps + wib) * PPW;
   const int t = w0 + lane;
-  const bool valid = t < n;
+  const bool valid = lane < PPW && t < n;
   const uint32_t ph = ctl->phase & 1u, lph = ctl->lphase & 1u;
   const uint32_t stamp_now = (uint32_t)ctl->step, stamp_new = stamp_now + 1u;
   const Rec* P = static_cast<const Rec*>(buf_of(sb.P, ph));
@@ -131,7 +115,7 @@ k_pairs(Ctl* ctl, Params p, StateBufs sb, Lists L, PairOut<typename Pol::T>* res
       if (e < Eu) {
         int lo = 0;
 #pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
+        for (int step = PPW / 2; step > 0; step >>= 1)
           if (seg[lo + step] <= e) lo += step;
         tl = lo;
         const uint32_t local = e - seg[tl];
@@ -174,33 +158,40 @@ k_pairs(Ctl* ctl, Params p, StateBufs sb, Lists L, PairOut<typename Pol::T>* res
   count_and_flag(ctl, npair, 0u, false, false);
 }
 
-// Per particle: the pair sums over the touched entries in list order, then
-// mesh contacts and integration; the touch mask is cleared for the next step.
-template <typename Pol, int MinBlocks>
-__global__ void __launch_bounds__(128, MinBlocks)
+// Per particle: the pair sums over the touched entries in list order (the
+// touch mask is cleared for the next step), then the warp's mesh contacts, 32
+// candidates at a time, then integration.  Taking a warp's candidates together
+// instead of each particle its own one by one matters in double precision: a
+// warp instruction costs the FP64 pipe the same whatever the lanes in use.
+template <typename Pol, int Warps, int PPW>
+__global__ void __launch_bounds__(32 * Warps, scaled_blocks(Pol::kMinBlocks, Warps))
 k_gather(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh,
          const PairOut<typename Pol::T>* res, unsigned long long* touch, double* forces) {
   using Rec = typename Pol::Rec;
   using CT = typename Pol::T;
+  __shared__ uint32_t seg_s[Warps][33];
+  __shared__ CT contrib_s[Warps][32][6];
   if (step_idle(ctl)) return;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = t < p.n;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int w0 = (blockIdx.x * Warps + wib) * PPW;
+  const int t = w0 + lane;
+  const bool valid = lane < PPW && t < p.n;
   const uint32_t ph = ctl->phase & 1u, lph = ctl->lphase & 1u;
   const uint32_t stamp_now = (uint32_t)ctl->step, stamp_new = stamp_now + 1u;
   const ListBuf lb = list_of(L, lph);
-  uint32_t nmesh = 0;
-  bool disp = false, bad = false;
+  const Rec* P = static_cast<const Rec*>(buf_of(sb.P, ph));
+  const Rec* V = static_cast<const Rec*>(buf_of(sb.V, ph));
+  const Rec* W = static_cast<const Rec*>(buf_of(sb.W, ph));
+  uint32_t nmesh = 0, ntc = 0;
+  typename Pol::Acc acc;
+  acc.zero();
   if (valid) {
-    const Rec* P = static_cast<const Rec*>(buf_of(sb.P, ph));
-    const Rec* V = static_cast<const Rec*>(buf_of(sb.V, ph));
-    const Rec* W = static_cast<const Rec*>(buf_of(sb.W, ph));
     const uint32_t meta = lb.meta[t];
     const uint32_t nlow = (meta >> 8) & 0xffu;
     const uint32_t off = lb.offs[t];
+    ntc = (meta >> 16) & 0xffu;
     unsigned long long m = touch[t];
     if (m) touch[t] = 0ull;
-    typename Pol::Acc acc;
-    acc.zero();
     CT c6[6];
     while (m) {
       const uint32_t k = (uint32_t)(__ffsll((long long)m) - 1);
@@ -210,22 +201,41 @@ k_gather(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh,
       get_out(res + e, !lower, c6);
       acc.add(c6);
     }
-    Pol::finish(p, sb, ph, lb, mesh, pose_at(mesh, ctl->step), t, (meta >> 16) & 0xffu, true, P[t], V[t], W[t], acc,
-                stamp_now, stamp_new, forces, nmesh, disp, bad);
   }
+  mesh_phase<Pol, PPW>(ctl, p, mesh, lb, P, V, W, seg_s[wib], contrib_s[wib], w0, ntc, stamp_now,
+                       stamp_new, acc, nmesh);
+  bool disp = false, bad = false;
+  if (valid) Pol::finish(p, sb, ph, lb, t, P[t], V[t], W[t], acc, forces, disp, bad);
   count_and_flag(ctl, 0u, nmesh, disp, bad);
 }
 
-template <typename Pol, int PairMinBlocks, int GatherMinBlocks>
-void launch_step_pairs(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
-                       MeshDev mesh, double* forces) {
+template <typename Pol, int Warps, int PPW>
+void launch_step_pairs_as(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
+                          MeshDev mesh, double* forces) {
   using Out = PairOut<typename Pol::T>;
   Out* res = static_cast<Out*>(p.pair_res);
-  k_pairs<Pol, PairMinBlocks>
-      <<<(unsigned)((p.n + 32 * kPairWarps - 1) / (32 * kPairWarps)), 32 * kPairWarps, 0, st>>>(
-          ctl, p, sb, L, res, p.pair_touch);
-  k_gather<Pol, GatherMinBlocks><<<(unsigned)((p.n + 127) / 128), 128, 0, st>>>(
-      ctl, p, sb, L, mesh, res, p.pair_touch, forces);
+  const unsigned nb = (unsigned)((p.n + PPW * Warps - 1) / (PPW * Warps));
+  k_pairs<Pol, Warps, PPW><<<nb, 32 * Warps, 0, st>>>(ctl, p, sb, L, res, p.pair_touch);
+  k_gather<Pol, Warps, PPW>
+      <<<nb, 32 * Warps, 0, st>>>(ctl, p, sb, L, mesh, res, p.pair_touch, forces);
+}
+
+// Small scenes spread their few warps over the SMs: an SM's FP64 pipe takes 16
+// cycles for a warp instruction, so the warps of one block wait for each other
+// while other SMs idle, and a warp with fewer particles has fewer batches in its
+// chain.  Measured (GB300, both kernels with ~4 us of event overhead, us, blocks
+// of one warp of 8 / 16 / 32 particles; 4 warps of 32): box n = 1,000 57 / 55 /
+// 76; 78, drum n = 3,000 61 / 96 / 135; 143, 20,000 158 / 139 / 150; 164, 200,000
+// 1147 / 813 / 623; 623.
+template <typename Pol>
+void launch_step_pairs(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
+                       MeshDev mesh, double* forces) {
+  if (p.n <= 8192)
+    launch_step_pairs_as<Pol, 1, 8>(st, ctl, p, sb, L, mesh, forces);
+  else if (p.n <= 40960)
+    launch_step_pairs_as<Pol, 1, 16>(st, ctl, p, sb, L, mesh, forces);
+  else
+    launch_step_pairs_as<Pol, 4, 32>(st, ctl, p, sb, L, mesh, forces);
 }
 
 }  // namespace dem

@@ -1,7 +1,7 @@
 // Warp-cooperative step kernel shared by both precisions.
 //
-// A warp owns 32 consecutive particle slots.  Their list entries are
-// contiguous in the CSR list, so:
+// A warp owns 32 consecutive particle slots (16 or 8 in small scenes, see
+// particles_per_warp).  Their list entries are contiguous in the CSR list, so:
 //   A. the lanes walk the warp's flattened entries 32 at a time (coalesced
 //      list reads), pre-test each pair for overlap with a cheap conservative
 //      test, and append the candidates (entry code and partner slot) to a
@@ -59,8 +59,65 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
   return v;
 }
 
-template <typename Pol, int Warps, bool Pose>
-__global__ void __launch_bounds__(32 * Warps, (Pol::kMinBlocks * 4 / Warps > 0 ? Pol::kMinBlocks * 4 / Warps : 1))
+// The particle-element contacts of a warp's particles (lane l < PPW owns slot
+// w0 + l with nt_l candidates), 32 candidates at a time (all lanes busy), then
+// ordered sums: every owner adds the touching contacts of its particle to its
+// sums in candidate (element index) order.  seg, contrib: shared memory of the
+// warp.
+template <typename Pol, int PPW>
+__device__ __forceinline__ void mesh_phase(const Ctl* ctl, const Params& p, const MeshDev& mesh,
+                                           const ListBuf& lb, const typename Pol::Rec* P,
+                                           const typename Pol::Rec* V,
+                                           const typename Pol::Rec* W, uint32_t* seg,
+                                           typename Pol::T (*contrib)[6], int w0, uint32_t nt_l,
+                                           uint32_t stamp_now, uint32_t stamp_new,
+                                           typename Pol::Acc& acc, uint32_t& nmesh) {
+  using CT = typename Pol::T;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const uint32_t mincl = warp_incl_scan(nt_l);
+  __syncwarp();
+  seg[lane + 1] = mincl;
+  if (lane == 0) seg[0] = 0;
+  const uint32_t Mt = __shfl_sync(full, mincl, 31);
+  __syncwarp();
+  const uint32_t my_a = seg[lane], my_b = seg[lane + 1];
+  for (uint32_t c0 = 0; c0 < Mt; c0 += 32) {
+    const uint32_t c = c0 + lane;
+    CT c6[6] = {CT(0), CT(0), CT(0), CT(0), CT(0), CT(0)};
+    bool hit = false;
+    if (c < Mt) {
+      int lo = 0;
+#pragma unroll
+      for (int step = PPW / 2; step > 0; step >>= 1)
+        if (seg[lo + step] <= c) lo += step;
+      const int tl = lo;
+      hit = Pol::mesh_contact(p, mesh, lb, w0 + tl, (int)(c - seg[tl]),
+                              pose_at(mesh, ctl->step), P[w0 + tl], V[w0 + tl], W[w0 + tl],
+                              stamp_now, stamp_new, c6);
+      if (hit) ++nmesh;
+    }
+    const unsigned hm = __ballot_sync(full, hit);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) contrib[lane][k] = c6[k];
+    __syncwarp();
+    const uint32_t a = my_a > c0 ? my_a : c0;
+    const uint32_t b = my_b < c0 + 32 ? my_b : c0 + 32;
+    for (uint32_t jj = a; jj < b; ++jj)
+      if (hm >> (jj - c0) & 1u) acc.add(contrib[jj - c0]);
+    __syncwarp();
+  }
+}
+
+// Resident blocks per SM of a kernel of `warps` warps per block, for a bound
+// stated for 4-warp blocks (at most the 32 blocks an SM holds).
+constexpr int scaled_blocks(int min_blocks4, int warps) {
+  const int b = min_blocks4 * 4 / warps;
+  return b < 1 ? 1 : (b > 32 ? 32 : b);
+}
+
+template <typename Pol, int Warps, int PPW, bool Pose>
+__global__ void __launch_bounds__(32 * Warps, scaled_blocks(Pol::kMinBlocks, Warps))
 k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* forces, int npose) {
   using Rec = typename Pol::Rec;
   using Hist = typename Pol::Hist;
@@ -76,9 +133,9 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   WarpScratch<CT>& S = smem[wib];
   const int n = p.n;
-  const int w0 = (((int)blockIdx.x - (Pose ? npose : 0)) * Warps + wib) * 32;
+  const int w0 = (((int)blockIdx.x - (Pose ? npose : 0)) * Warps + wib) * PPW;
   const int t = w0 + lane;
-  const bool valid = t < n;
+  const bool valid = lane < PPW && t < n;
   const uint32_t ph = ctl->phase & 1u, lph = ctl->lphase & 1u;
   const uint32_t stamp_now = (uint32_t)ctl->step;
   const uint32_t stamp_new = stamp_now + 1u;
@@ -124,7 +181,7 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
         // the particle owning entry e: largest tl with seg[tl] <= e
         int lo = 0;
 #pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
+        for (int step = PPW / 2; step > 0; step >>= 1)
           if (S.seg[lo + step] <= e) lo += step;
         tl = lo;
         const uint32_t k = e - S.seg[tl];
@@ -181,7 +238,7 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
       const uint32_t last = (i0 + 32 < qn ? i0 + 32 : qn) - 1u;
       int pa = 0, pb = 0;
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
+      for (int step = PPW / 2; step > 0; step >>= 1) {
         if (S.istart[pa + step] <= i0) pa += step;
         if (S.istart[pb + step] <= last) pb += step;
       }
@@ -202,73 +259,59 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
   __syncwarp();
   acc.set(S.acc_h[lane], S.acc_l[lane]);
 
-  // M: particle-element contacts of the warp's particles, 32 candidates at a
-  // time (all lanes busy), then ordered sums as in B: every lane adds the
-  // touching contacts of its own particle in candidate (element index) order
+  // M: particle-element contacts of the warp's particles
   uint32_t nmesh = 0;
-  {
-    const uint32_t nt_l = valid ? (meta >> 16) & 0xffu : 0u;
-    const uint32_t mincl = warp_incl_scan(nt_l);
-    __syncwarp();
-    S.seg[lane + 1] = mincl;
-    if (lane == 0) S.seg[0] = 0;
-    const uint32_t Mt = __shfl_sync(full, mincl, 31);
-    __syncwarp();
-    const uint32_t my_a = S.seg[lane], my_b = S.seg[lane + 1];
-    for (uint32_t c0 = 0; c0 < Mt; c0 += 32) {
-      const uint32_t c = c0 + lane;
-      CT c6[6] = {CT(0), CT(0), CT(0), CT(0), CT(0), CT(0)};
-      bool hit = false;
-      if (c < Mt) {
-        int lo = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
-          if (S.seg[lo + step] <= c) lo += step;
-        const int tl = lo;
-        hit = Pol::mesh_contact(p, mesh, lb, w0 + tl, (int)(c - S.seg[tl]),
-                                pose_at(mesh, ctl->step), P[w0 + tl], V[w0 + tl], W[w0 + tl], stamp_now, stamp_new, c6);
-        if (hit) ++nmesh;
-      }
-      const unsigned hm = __ballot_sync(full, hit);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) S.contrib[lane][k] = c6[k];
-      __syncwarp();
-      const uint32_t a = my_a > c0 ? my_a : c0;
-      const uint32_t b = my_b < c0 + 32 ? my_b : c0 + 32;
-      for (uint32_t jj = a; jj < b; ++jj)
-        if (hm >> (jj - c0) & 1u) acc.add(S.contrib[jj - c0]);
-      __syncwarp();
-    }
-  }
+  mesh_phase<Pol, PPW>(ctl, p, mesh, lb, P, V, W, S.seg, S.contrib, w0,
+                       valid ? (meta >> 16) & 0xffu : 0u, stamp_now, stamp_new, acc, nmesh);
 
   // C: integration of the lane's own particle
   bool disp = false, bad = false;
   if (valid)
-    Pol::finish(p, sb, ph, lb, mesh, 0u, t, (meta >> 16) & 0xffu, false, P[t], V[t],
-                W[t], acc, stamp_now, stamp_new, forces, nmesh, disp, bad);
+    Pol::finish(p, sb, ph, lb, t, P[t], V[t], W[t], acc, forces, disp, bad);
 
   count_and_flag(ctl, npair, nmesh, disp, bad);
 }
 
-template <typename Pol, int Warps>
+template <typename Pol, int Warps, int PPW, bool Pose>
 void launch_step_warp_as(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
                          MeshDev mesh, double* forces, bool pose) {
-  constexpr int kThreads = 32 * Warps;
-  const int npose = pose ? (mesh.nt + kThreads - 1) / kThreads : 0;
-  const unsigned nb = (unsigned)((p.n + kThreads - 1) / kThreads + npose);
-  if (pose)
-    k_step_warp<Pol, Warps, true><<<nb, kThreads, 0, st>>>(ctl, p, sb, L, mesh, forces, npose);
-  else
-    k_step_warp<Pol, Warps, false><<<nb, kThreads, 0, st>>>(ctl, p, sb, L, mesh, forces, 0);
+  const int npose = pose ? (mesh.nt + 32 * Warps - 1) / (32 * Warps) : 0;
+  const unsigned nb = (unsigned)((p.n + PPW * Warps - 1) / (PPW * Warps) + npose);
+  k_step_warp<Pol, Warps, PPW, Pose>
+      <<<nb, 32 * Warps, 0, st>>>(ctl, p, sb, L, mesh, forces, npose);
+}
+
+// Particles per warp.  A warp takes its particles' entries and contacts 32 at
+// a time, one batch after the other; a small scene has too few warps to hide
+// those chains (20,000 particles: 4 warps of 32 an SM), so its warps own fewer
+// particles.  The price is lanes left idle: the integration uses only as many
+// lanes as particles.  Measured (GB300, step kernel with ~4 us of event
+// overhead, us, warps of 8 / 16 / 32 particles): DEM_MIXED drum n = 3,000 12.4
+// / 18.4 / 28.6, 20,000 16.4 / 20.5 / 28.7, 60,000 32.8 / 26.6 / 30.7, 150,000
+// 63.5 / 51.2 / 43.0, 1,000,000 346 / 254 / 215; DEM_MIXED64 column n = 3,000
+// 18.5 / 20.5 / 22.5, 20,000 28.7 / 24.6 / 26.6, 200,000 174 / 108 / 78.  Results
+// do not depend on it.
+inline int particles_per_warp(const Params& p) {
+  if (p.n <= (p.mixed ? 32768 : 8192)) return 8;
+  return p.n <= (p.mixed ? 81920 : 40960) ? 16 : 32;
 }
 
 template <typename Pol>
 void launch_step_warp(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
                       MeshDev mesh, double* forces, bool pose) {
-  if (p.step_warps == 8)
-    launch_step_warp_as<Pol, 8>(st, ctl, p, sb, L, mesh, forces, pose);
+  const int ppw = particles_per_warp(p);
+  if (ppw == 8)
+    launch_step_warp_as<Pol, 4, 8, true>(st, ctl, p, sb, L, mesh, forces, pose);
+  else if (ppw == 16)
+    launch_step_warp_as<Pol, 4, 16, true>(st, ctl, p, sb, L, mesh, forces, pose);
+  else if (p.step_warps == 8 && pose)
+    launch_step_warp_as<Pol, 8, 32, true>(st, ctl, p, sb, L, mesh, forces, true);
+  else if (p.step_warps == 8)
+    launch_step_warp_as<Pol, 8, 32, false>(st, ctl, p, sb, L, mesh, forces, false);
+  else if (pose)
+    launch_step_warp_as<Pol, 4, 32, true>(st, ctl, p, sb, L, mesh, forces, true);
   else
-    launch_step_warp_as<Pol, 4>(st, ctl, p, sb, L, mesh, forces, pose);
+    launch_step_warp_as<Pol, 4, 32, false>(st, ctl, p, sb, L, mesh, forces, false);
 }
 
 }  // namespace dem

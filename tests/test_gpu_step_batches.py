@@ -56,3 +56,22 @@ def test_same_bits_however_the_steps_are_cut(dem, monkeypatch, scene, precision)
     st, _ = run(dem, s, precision, [200])
     for k in ref:
         assert np.array_equal(ref[k], st[k]), k
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2], ids=["fp64", "mixed", "mixed64"])
+@pytest.mark.parametrize("n", [1, 7, 9, 777])
+def test_same_bits_for_any_number_of_rows(dem, precision, n):
+    # the step kernels give a warp 8, 16 or 32 particles by the number of rows
+    # of the scene; rows that await spawning (none is spawned here) change that
+    # number and nothing else
+    s = scenes.drum_scene(n=n, seed=6, n_theta=32, n_rings=4, nn_dist=2.0e-3, radius=0.018,
+                          speed=0.5)
+    ref, stats = run(dem, s, precision, [60])
+    for rows in (8193, 32769, 40961, 81921):
+        s["spawn"] = dict(n_max=rows, lo=(0, 0, 0), hi=(0, 0, 0), r_min=1e-3, r_max=1e-3,
+                          attempts=0)
+        st, other = run(dem, s, precision, [60])
+        assert other["pair_contacts"] == stats["pair_contacts"]
+        assert other["mesh_contacts"] == stats["mesh_contacts"]
+        for k in ref:
+            assert np.array_equal(ref[k], st[k][:n]), (rows, k)
