@@ -980,12 +980,12 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
   // one cell more than the grid: inactive particles (awaiting spawning)
   s->bb.cell_count = M.get<uint32_t>(ncells + 1);
   s->bb.cell_start = M.get<uint32_t>(ncells + 2);
-  s->bb.block_sums = M.get<uint32_t>(scan_block_sums_size(std::max<int64_t>(ncells + 1, n)) + 1);
+  s->bb.src = M.get<uint32_t>(n);
+  s->bb.block_sums = M.get<uint32_t>(
+      std::max(scan_block_sums_size(ncells + 1), list_block_sums_size(n)) + 1);
+  s->bb.scan_done = M.get<uint32_t>(1);
   s->bb.tmp_nbr = M.get<uint32_t>((size_t)p.cap * n);
-  s->bb.tmp_gid = M.get<uint32_t>((size_t)p.cap * n);
-  s->bb.tmp_hsrc = M.get<uint32_t>((size_t)p.cap * n);
   s->bb.tmp_cnt = M.get<uint32_t>(n);
-  s->bb.tmp_offs = M.get<uint32_t>(n + 1);
   if (p.record_forces) s->forces = M.get<double>(6 * (size_t)n);
   s->export_buf = M.get<double>(13 * (size_t)n);
   if (one_eval_per_pair(p)) {  // one evaluation per pair
@@ -995,7 +995,7 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
   if (has_mesh) {
     s->bb.tcell_count = M.get<uint32_t>(ncells);
     s->bb.tcell_start = M.get<uint32_t>(ncells + 1);
-    s->bb.tcell_overflow = M.get<uint32_t>(2);  // [1]: element lists of a still mesh built
+    s->bb.tcell_overflow = M.get<uint32_t>(1);
     // capacity: for every element, the cells of a cube around its bounding
     // ball grown by the reach (valid for any pose of a rigid mesh)
     const double reach = rmax + skin + 2.0 * p.list_margin;
@@ -1066,7 +1066,8 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
     p.mat_d = md;
   }
   if (M.failed) return fail(DEM_ERR_NOMEM);
-  if (has_mesh && cudaMemset(s->bb.tcell_overflow, 0, 2 * sizeof(uint32_t)) != cudaSuccess)
+  if (cudaMemset(s->bb.cell_count, 0, (ncells + 1) * sizeof(uint32_t)) != cudaSuccess ||
+      cudaMemset(s->bb.scan_done, 0, sizeof(uint32_t)) != cudaSuccess)
     return fail(DEM_ERR_CUDA);
   s->mesh.nv = s->nv;
   s->mesh.nt = s->nt;
@@ -1094,9 +1095,8 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
         cudaMemcpy(s->mesh.rad, et.rad.data(), s->nt * sizeof(double), cudaMemcpyHostToDevice))
       return fail(DEM_ERR_CUDA);
   }
-  // kernels per step: mesh pose, [decide], rebuild (prep, clear, count, 3 scan,
-  // scatter, cell sort, permute, [mesh: clear, count, 3 scan, check, clear, fill,
-  // sort], list build, 3 scan, compact, end), step, advance -- see dem_get_stats
+  // kernels of a rebuild: count, 2 scan, scatter, permute, list build, offsets,
+  // compact, [mirror], end -- see dem_get_stats
   {
     // capacity rows: the given particles, then inactive rows (radius 0)
     std::vector<double> R(n, 0.0), x(3 * n, 0.0), v(3 * n, 0.0), w(3 * n, 0.0), q(4 * n, 0.0);
@@ -1121,6 +1121,7 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
   // poses of steps 0 and 1 (a static mesh keeps them)
   launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 0);
   launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 1);
+  if (has_mesh) launch_mesh_cells(s->stream, s->ctl, s->p, s->bb, s->mesh);
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) return fail(DEM_ERR_CUDA);
   // capture and instantiate the step graphs now, so that no dem_step call
   // pays for it on the host while the device waits; a failure here leaves
@@ -1291,7 +1292,7 @@ int dem_get_stats(dem_scene* s, dem_stats* out) {
   out->status = (int32_t)c.status;
   out->active = c.n_active;
   out->capacity = s->n;
-  const int32_t rebuild_launches = 15 + (s->nt > 0 ? 9 : 0) + (s->p.pair_res ? 1 : 0);
+  const int32_t rebuild_launches = 9 + (s->p.pair_res ? 1 : 0);
   const int32_t base = (s->static_mesh || step_poses(s->p) ? 0 : 1) + 2 +
                        (s->p.sp_attempts > 0 ? 1 : 0) + (s->p.pair_res ? 1 : 0);
   if (s->conditional_graphs) {

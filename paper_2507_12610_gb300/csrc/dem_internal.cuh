@@ -189,28 +189,24 @@ struct MeshDev {
   int32_t nv, nt;
 };
 
-constexpr uint32_t kNoHist = 0xffffffffu;  // no history record to carry over
-
 // Binning scratch.
 struct BinBuf {
   uint32_t* key;        // [n] cell of each slot (current order)
   uint32_t* local;      // [n] arrival index within its cell
-  uint32_t* cell_count; // [ncells]
+  uint32_t* cell_count; // [ncells + 1], zero between rebuilds (the scan clears it)
   uint32_t* cell_start; // [ncells + 1]
-  uint32_t* order;      // [n] old slot of each new slot
+  uint32_t* order;      // [n] old slots by cell, in arrival order within a cell
+  uint32_t* src;        // [n] old slot of each new slot
   uint32_t* block_sums; // scan partials
+  uint32_t* scan_done;  // [1] blocks of a scan that have finished (zero between scans)
   uint32_t* tmp_nbr;    // [cap][n] candidates of the list being built (slot order)
-  uint32_t* tmp_gid;    // [cap][n] their caller indices
-  uint32_t* tmp_hsrc;   // [cap][n] index of the entry's history record in the
-                        //   previous list, or kNoHist
-  uint32_t* tmp_cnt;    // [n] their counts
-  uint32_t* tmp_offs;   // [n + 1] exclusive prefix of the counts
+  uint32_t* tmp_cnt;    // [n] their counts | element candidates << 16
   // triangle cell lists
   uint32_t* tcell_count;  // [ncells]
   uint32_t* tcell_start;  // [ncells + 1]
   uint32_t* tcell_tri;    // [tcap]
   uint32_t tcap;
-  uint32_t* tcell_overflow;
+  uint32_t* tcell_overflow;  // [1] entries the lists would need beyond tcap, or 0
 };
 
 // Both parities of the double-buffered data.  Kernels pick the current one
@@ -294,9 +290,13 @@ void launch_set_left(cudaStream_t st, Ctl* ctl, int64_t left);
 void launch_decide(cudaStream_t st, const Ctl* ctl, cudaGraphConditionalHandle h);
 void launch_again(cudaStream_t st, const Ctl* ctl, cudaGraphConditionalHandle h);
 
+// The element cell lists (once per scene, after the first upload).
+void launch_mesh_cells(cudaStream_t st, Ctl* ctl, const Params& p, BinBuf bb, MeshDev mesh);
+
 // Scan of a u32 array (exclusive) on the device; early-exits unless ctl->rebuild.
-void launch_scan(cudaStream_t st, const Ctl* ctl, const uint32_t* in, uint32_t* out, int64_t n,
-                 uint32_t* block_sums);
+void launch_scan(cudaStream_t st, const Ctl* ctl, uint32_t* in, uint32_t* out, int64_t n,
+                 uint32_t* block_sums, uint32_t* done, bool clear);
 int64_t scan_block_sums_size(int64_t n);
+int64_t list_block_sums_size(int64_t n);
 
 }  // namespace dem
