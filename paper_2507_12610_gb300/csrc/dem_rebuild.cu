@@ -25,6 +25,7 @@ namespace dem {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kTotalSlots = 128;  // slots per entry of the list totals
 
 __device__ __forceinline__ bool rebuilding(const Ctl* ctl) {
   return ctl->rebuild != 0 && ctl->status == 0;
@@ -94,7 +95,6 @@ k_bin_count(Ctl* ctl, Params p, StateBufs sb, BinBuf bb, Lists L) {
         ctl->rot_c = cos(th);
         ctl->rot_s = sin(th);
       }
-      ctl->list_entries = 0;
       ctl->mesh_candidates = 0;
       ctl->max_list_len = 0;
       if (p.n_tri > 0 && *bb.tcell_overflow) set_status(ctl, DEM_ERR_CAPACITY);
@@ -145,6 +145,7 @@ k_permute(const Ctl* ctl, Params p, BinBuf bb, StateBufs sb, Lists L) {
   const uint32_t* gid_old = list_of(L, lph).gid;
   uint32_t* gid_new = list_of(L, lph ^ 1u).gid;
   float4* posf_new = list_of(L, lph ^ 1u).posf;
+  if (a % kTotalSlots == 0) bb.block_sums[a / kTotalSlots] = 0u;  // for the list build
   const uint32_t s = bb.order[a];
   const uint32_t c = bb.key[s], g = gid_old[s];
   uint32_t t = (uint32_t)a;  // inactive particles arrived in caller order
@@ -302,119 +303,139 @@ k_tri_cell_sort(Params p, BinBuf bb) {
 // history over from the particle's previous list.  k_list_compact sorts the
 // pair list and carries the pairs' history over.
 //
-// One thread per slot; the candidate positions come through L1 (a block's
-// slots are neighbours in cell order, so they read the same cells).  Staging
-// the neighbour rows of a block in shared memory first was measured slower
-// (the threads of a block that spans two rows of cells wait for each other).
-constexpr int kBuildThreads = 128;
+// G lanes share a particle and take a row's candidates G at a time; the first
+// candidates of three rows are loaded together.  Small scenes are bound by a
+// particle's chain of ~76 tests, so more lanes share it; large ones by the
+// instructions, of which groups need more (lanes idle at the ends of rows).
+// Measured (GB300, us, G = 1 / 2 / 4 / 8): box n = 1,000 12.5 / 9.3 / 7.4 / 7.1
+// (15.7 with one lane a particle and no loads ahead), drum n = 20,000 30 / 19 /
+// 13.4 / 15.9 (32), 200,000 51 / 48 / 56 / -, 1,000,000 181 / 207 / 257 / -.
+constexpr int kBuildThreads = 256;
 
-template <typename Hist>
+template <typename Hist, int G>
 __global__ void __launch_bounds__(kBuildThreads)
 k_list_build(Ctl* ctl, Params p, BinBuf bb, Lists L, MeshDev mesh) {
-  __shared__ uint32_t total_s[kBuildThreads / 32];
   if (!rebuilding(ctl)) return;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane & (G - 1), g0 = lane & ~(G - 1);
+  const unsigned below = (1u << sub) - 1u, group = (1u << G) - 1u;
+  const int t = (int)(blockIdx.x * (kBuildThreads / G) + threadIdx.x / G);
   const int n = p.n;
   const ListBuf lo = list_of(L, ctl->lphase & 1u);
   const ListBuf ln = list_of(L, (ctl->lphase & 1u) ^ 1u);
   const float4 X = t < n ? ln.posf[t] : make_float4(0.f, 0.f, 0.f, 0.f);
+  const bool on = X.w != 0.f;  // (inactive: no list, no mesh candidates)
+  const int3 c = cell_coords(p, X.x, X.y, X.z);
   int cnt = 0, ntc = 0;
   bool overflow = false;
-  if (X.w != 0.f) {  // (inactive: no list, no mesh candidates)
-    const int3 c = cell_coords(p, X.x, X.y, X.z);
-    // the cells of a row along x are consecutive in the grid, so the three
-    // cells x-1 .. x+1 of a neighbour row are one range of slots: 9 ranges
-    const int x0 = max(c.x - 1, 0), x1 = min(c.x + 1, p.nc[0] - 1);
-    for (int dz = -1; dz <= 1; ++dz) {
-      const int cz = c.z + dz;
-      if (cz < 0 || cz >= p.nc[2]) continue;
-      for (int dy = -1; dy <= 1; ++dy) {
-        const int cy = c.y + dy;
-        if (cy < 0 || cy >= p.nc[1]) continue;
-        const uint32_t a = bb.cell_start[cell_index(p, make_int3(x0, cy, cz))];
-        const uint32_t b = bb.cell_start[cell_index(p, make_int3(x1, cy, cz)) + 1];
-        for (uint32_t u = a; u < b; ++u) {
-          const float4 Y = ln.posf[u];
-          const float ddx = X.x - Y.x, ddy = X.y - Y.y, ddz = X.z - Y.z;
-          const float cut = X.w + Y.w + p.skin + p.list_margin;
-          if (ddx * ddx + ddy * ddy + ddz * ddz < cut * cut && u != (uint32_t)t) {
-            if (cnt < p.cap)
-              bb.tmp_nbr[(size_t)cnt++ * n + t] = u;
-            else
-              overflow = true;
-          }
+  // the cells of a row along x are consecutive in the grid, so the three
+  // cells x-1 .. x+1 of a neighbour row are one range of slots: 9 ranges, three
+  // (one z) at a time
+  const int x0 = max(c.x - 1, 0), x1 = min(c.x + 1, p.nc[0] - 1);
+#pragma unroll 1
+  for (int dz = -1; dz <= 1; ++dz) {
+    const int cz = c.z + dz;
+    uint32_t ua[3], ub[3];
+    float4 Y[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int cy = c.y + r - 1;
+      const bool in = on && cz >= 0 && cz < p.nc[2] && cy >= 0 && cy < p.nc[1];
+      ua[r] = in ? bb.cell_start[cell_index(p, make_int3(x0, cy, cz))] + sub : 0u;
+      ub[r] = in ? bb.cell_start[cell_index(p, make_int3(x1, cy, cz)) + 1] : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+      if (ua[r] < ub[r]) Y[r] = ln.posf[ua[r]];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      bool more = __any_sync(full, ua[r] < ub[r]);
+      while (more) {
+        const uint32_t u = ua[r];
+        bool hit = false;
+        if (u < ub[r]) {
+          const float ddx = X.x - Y[r].x, ddy = X.y - Y[r].y, ddz = X.z - Y[r].z;
+          const float cut = X.w + Y[r].w + p.skin + p.list_margin;
+          hit = ddx * ddx + ddy * ddy + ddz * ddz < cut * cut && u != (uint32_t)t;
         }
+        ua[r] = u + G;
+        if (ua[r] < ub[r]) Y[r] = ln.posf[ua[r]];
+        more = __any_sync(full, ua[r] < ub[r]);
+        const unsigned m = (__ballot_sync(full, hit) >> g0) & group;
+        if (hit) {
+          const int at = cnt + __popc(m & below);
+          if (at < p.cap)
+            bb.tmp_nbr[(size_t)at * n + t] = u;
+          else
+            overflow = true;
+        }
+        cnt += __popc(m);
       }
     }
-    // triangle candidates (fixed capacity per particle), history carried over
-    if (mesh.nt > 0) {
-      // the element list of the particle's cell in the mesh's frame
-      int3 cm = c;
-      if (p.omega_norm > 0.0) {
-        const V3<float> qm = to_mesh_frame(p, mk(X.x, X.y, X.z), (float)ctl->rot_c,
-                                           (float)ctl->rot_s);
-        cm = cell_coords(p, qm.x, qm.y, qm.z);
-      }
-      const uint32_t cell = cell_index(p, cm);
-      const uint32_t a = bb.tcell_start[cell], b = min(bb.tcell_start[cell + 1], bb.tcap);
-      const uint32_t stamp_now = (uint32_t)ctl->step;  // records written in the previous step
-      const uint32_t pose = pose_at(mesh, ctl->step);
-      const Hist* hpm_o = static_cast<const Hist*>(lo.hpm);
-      Hist* hpm_n = static_cast<Hist*>(ln.hpm);
-      uint32_t s = 0;
-      int nt_o = 0, ko2 = 0;
-      if (a < b) {
-        s = bb.src[t];
-        nt_o = (int)((lo.meta[s] >> 16) & 0xffu);
-      }
-      const V3<float> q = mk(X.x, X.y, X.z);
-      for (uint32_t i = a; i < b; ++i) {
-        const uint32_t k = bb.tcell_tri[i];
+  }
+  // triangle candidates (fixed capacity per particle), history carried over:
+  // the group takes the elements of the cell's list G at a time, in order
+  if (mesh.nt > 0) {
+    // the element list of the particle's cell in the mesh's frame
+    int3 cm = c;
+    if (p.omega_norm > 0.0) {
+      const V3<float> qm = to_mesh_frame(p, mk(X.x, X.y, X.z), (float)ctl->rot_c,
+                                         (float)ctl->rot_s);
+      cm = cell_coords(p, qm.x, qm.y, qm.z);
+    }
+    const uint32_t cell = cell_index(p, cm);
+    uint32_t i = on ? bb.tcell_start[cell] + sub : 0u;
+    const uint32_t b = on ? min(bb.tcell_start[cell + 1], bb.tcap) : 0u;
+    const uint32_t stamp_now = (uint32_t)ctl->step;  // records written in the previous step
+    const uint32_t pose = pose_at(mesh, ctl->step);
+    const Hist* hpm_o = static_cast<const Hist*>(lo.hpm);
+    Hist* hpm_n = static_cast<Hist*>(ln.hpm);
+    for (; __any_sync(full, i < b); i += G) {
+      bool hit = false;
+      uint32_t k = 0;
+      if (i < b) {
+        k = bb.tcell_tri[i];
         const float4* v4 = mesh.curf + 4 * (size_t)(pose + k);
         const float4 A = v4[0], B = v4[1], C = v4[2], D = v4[3];
+        const V3<float> q = mk(X.x, X.y, X.z);
         const V3<float> y = closest_point_element(q, mk(A.x, A.y, A.z), mk(B.x, B.y, B.z),
                                                   mk(C.x, C.y, C.z), mk(D.x, D.y, D.z), (int)A.w);
         const V3<float> d = q - y;
         const float cut = X.w + (float)mesh.rad[k] + p.skin + p.list_margin;
-        if (dot(d, d) >= cut * cut) continue;
-        if (ntc >= p.capm) {
-          overflow = true;
-          continue;
-        }
-        ln.tric[(size_t)ntc * n + t] = k;
-        while (ko2 < nt_o && lo.tric[(size_t)ko2 * n + s] < k) ++ko2;
-        if (ko2 < nt_o && lo.tric[(size_t)ko2 * n + s] == k) {
-          const Hist h = hpm_o[(size_t)ko2 * n + s];
-          if (h.stamp == stamp_now) hpm_n[(size_t)ntc * n + t] = h;
-        }
-        ++ntc;
+        hit = dot(d, d) < cut * cut;
       }
+      const unsigned m = (__ballot_sync(full, hit) >> g0) & group;
+      if (hit) {
+        const int at = ntc + __popc(m & below);
+        if (at < p.capm) {
+          ln.tric[(size_t)at * n + t] = k;
+          // the particle's previous list (ascending, a few elements)
+          const uint32_t s = bb.src[t];
+          const int nt_o = (int)((lo.meta[s] >> 16) & 0xffu);
+          int j = 0;
+          while (j < nt_o && lo.tric[(size_t)j * n + s] < k) ++j;
+          if (j < nt_o && lo.tric[(size_t)j * n + s] == k) {
+            const Hist h = hpm_o[(size_t)j * n + s];
+            if (h.stamp == stamp_now) hpm_n[(size_t)at * n + t] = h;
+          }
+        } else {
+          overflow = true;
+        }
+      }
+      ntc += __popc(m);
     }
   }
   if (overflow) set_status(ctl, DEM_ERR_CAPACITY);
-  if (t < n) bb.tmp_cnt[t] = (uint32_t)cnt | ((uint32_t)ntc << 16);
-  // counters, one atomic a warp, and the block's entries for the offsets
-  const unsigned full = 0xffffffffu;
-  const int wid = threadIdx.x >> 5;
-  const uint32_t sum = __reduce_add_sync(full, (uint32_t)cnt);
-  const uint32_t sumt = __reduce_add_sync(full, (uint32_t)ntc);
-  const uint32_t most = __reduce_max_sync(full, (uint32_t)cnt);
-  if ((threadIdx.x & 31) == 0) {
-    total_s[wid] = sum;
-    if (sum) atomicAdd(&ctl->list_entries, sum);
-    if (sumt) atomicAdd(&ctl->mesh_candidates, sumt);
-    if (most) atomicMax(&ctl->max_list_len, most);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t total = 0;
-    for (int w = 0; w < kBuildThreads / 32; ++w) total += total_s[w];
-    bb.block_sums[blockIdx.x] = total;
-  }
+  cnt = min(cnt, p.cap);
+  if (sub == 0 && t < n) bb.tmp_cnt[t] = (uint32_t)cnt | ((uint32_t)min(ntc, p.capm) << 16);
+  // the warp's entries into the total of its kTotalSlots slots
+  const uint32_t sum = __reduce_add_sync(full, sub == 0 ? (uint32_t)cnt : 0u);
+  if (lane == 0 && sum) atomicAdd(&bb.block_sums[t / kTotalSlots], sum);
 }
 
-// Exclusive scan of the list build's block totals (one block, ascending), and
-// the total to offs[n].
+// Exclusive scan of the list build's totals (one block, ascending); the sum of
+// all to offs[n] and the control block.
 constexpr int kOffsetThreads = 1024;
 
 __device__ __forceinline__ uint32_t warp_scan_incl(uint32_t v) {
@@ -428,7 +449,7 @@ __device__ __forceinline__ uint32_t warp_scan_incl(uint32_t v) {
 }
 
 __global__ void __launch_bounds__(kOffsetThreads)
-k_list_offsets(const Ctl* ctl, Params p, BinBuf bb, Lists L, int nblocks) {
+k_list_offsets(Ctl* ctl, Params p, BinBuf bb, Lists L, int nblocks) {
   __shared__ uint32_t warp_s[kOffsetThreads / 32];
   if (!rebuilding(ctl)) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -456,14 +477,17 @@ k_list_offsets(const Ctl* ctl, Params p, BinBuf bb, Lists L, int nblocks) {
     carry += __shfl_sync(0xffffffffu, wtot, 31);
     __syncthreads();
   }
-  if (threadIdx.x == 0) list_of(L, (ctl->lphase & 1u) ^ 1u).offs[p.n] = carry;
+  if (threadIdx.x == 0) {
+    list_of(L, (ctl->lphase & 1u) ^ 1u).offs[p.n] = carry;
+    ctl->list_entries = carry;
+  }
 }
 
 // Sort the new pair lists by partner caller index into CSR form and copy each
 // pair's friction history record from the previous list where that list has
 // the pair and the contact touched in the previous step (with one evaluation
 // per pair only the entries of partners with a higher caller index hold
-// records).  A warp takes the entries of its 32 slots, kStage at a time: staged
+// records).  A warp takes the entries of its slots, kStage at a time: staged
 // in shared memory with their caller indices, each entry's place is its rank
 // among its particle's entries, and a binary search of the particle's previous
 // list (sorted the same way, a cache line or two) finds the old record.
@@ -472,31 +496,32 @@ k_list_offsets(const Ctl* ctl, Params p, BinBuf bb, Lists L, int nblocks) {
 // to 9, took a rebuild (with its launches) from 635 to 480 us on the
 // 1,000,000-sphere drum, from 315 to 170 us on the 200,000-sphere column and
 // from 128 to 66 us on the 1,000-sphere box.
-constexpr int kCompactWarps = kBuildThreads / 32;  // the list build's blocks
-constexpr uint32_t kStage = 512;                   // >= 64, the longest list
-
-template <typename Hist>
-__global__ void __launch_bounds__(32 * kCompactWarps)
+// Slots: 32 a warp, 8 in small scenes (fewer batches in a warp's chain: 23.4
+// -> 11.2 us at 20,000 spheres, 9.2 -> 6.4 us at 1,000).
+template <typename Hist, int Slots>
+__global__ void __launch_bounds__(32 * (kTotalSlots / Slots))
 k_list_compact(Ctl* ctl, Params p, BinBuf bb, Lists L) {
-  __shared__ uint32_t seg_s[kCompactWarps][33];
-  __shared__ uint32_t off_s[kCompactWarps][32];  // previous list: first entry
-  __shared__ uint32_t nold_s[kCompactWarps][32];  // and length
-  __shared__ uint32_t gid_s[kCompactWarps][32];
-  __shared__ uint32_t slot_s[kCompactWarps][kStage];
-  __shared__ uint32_t pgid_s[kCompactWarps][kStage];
-  __shared__ uint32_t total_s[kCompactWarps];
+  constexpr int kWarps = kTotalSlots / Slots;  // a block takes one of the list totals
+  constexpr uint32_t kStage = 16 * Slots;      // >= 64, the longest list
+  __shared__ uint32_t seg_s[kWarps][33];
+  __shared__ uint32_t off_s[kWarps][32];   // previous list: first entry
+  __shared__ uint32_t nold_s[kWarps][32];  // and length
+  __shared__ uint32_t gid_s[kWarps][32];
+  __shared__ uint32_t slot_s[kWarps][kStage];
+  __shared__ uint32_t pgid_s[kWarps][kStage];
+  __shared__ uint32_t total_s[kWarps];
   if (!rebuilding(ctl)) return;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int n = p.n;
-  const int w0 = (blockIdx.x * kCompactWarps + wib) * 32;
-  const int t = w0 + lane;
+  const int t = (blockIdx.x * kWarps + wib) * Slots + lane;
+  const bool own = lane < Slots && t < n;
   const ListBuf lo = list_of(L, ctl->lphase & 1u);
   const ListBuf ln = list_of(L, (ctl->lphase & 1u) ^ 1u);
   uint32_t* seg = seg_s[wib];
   uint32_t* slot = slot_s[wib];
   uint32_t* pgid = pgid_s[wib];
-  const uint32_t packed = t < n ? bb.tmp_cnt[t] : 0u;
+  const uint32_t packed = own ? bb.tmp_cnt[t] : 0u;
   const uint32_t cnt = packed & 0xffffu;
   const uint32_t incl = warp_scan_incl(cnt);
   seg[lane + 1] = incl;
@@ -513,18 +538,19 @@ k_list_compact(Ctl* ctl, Params p, BinBuf bb, Lists L) {
   nold_s[wib][lane] = nn_o;
   gid_s[wib][lane] = g_own;
   __syncthreads();
-  uint32_t base = bb.block_sums[blockIdx.x];  // first entry of slot w0
+  uint32_t base = bb.block_sums[blockIdx.x];  // first entry of the warp's first slot
   for (int w = 0; w < wib; ++w) base += total_s[w];
-  if (t < n) ln.offs[t] = base + incl - cnt;
+  if (own) ln.offs[t] = base + incl - cnt;
   const bool one_eval = p.pair_res != nullptr;
   const Hist* hpp_o = static_cast<const Hist*>(lo.hpp);
   Hist* hpp_n = static_cast<Hist*>(ln.hpp);
   const uint32_t stamp_now = (uint32_t)ctl->step;  // records written in the previous step
   uint32_t nlow = 0;
-  for (int a = 0; a < 32;) {
+  for (int a = 0; a < Slots;) {
     // slots a .. b-1: as many as the stage holds (at least one)
     const uint32_t first = seg[a];
-    const unsigned fit = __ballot_sync(full, lane >= a && seg[lane + 1] - first <= kStage);
+    const unsigned fit =
+        __ballot_sync(full, lane >= a && lane < Slots && seg[lane + 1] - first <= kStage);
     const int b = 32 - __clz((int)fit);
     if (lane >= a && lane < b) {
       const uint32_t at = seg[lane] - first;
@@ -542,7 +568,7 @@ k_list_compact(Ctl* ctl, Params p, BinBuf bb, Lists L) {
       // the slot owning the entry: largest tl with seg[tl] <= first + e
       int tl = 0;
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1)
+      for (int step = Slots / 2; step > 0; step >>= 1)
         if (seg[tl + step] <= first + e) tl += step;
       const uint32_t j0 = seg[tl] - first, j1 = seg[tl + 1] - first;
       const uint32_t g = pgid[e];
@@ -566,7 +592,14 @@ k_list_compact(Ctl* ctl, Params p, BinBuf bb, Lists L) {
     __syncwarp();
     a = b;
   }
-  if (t < n) ln.meta[t] = cnt | (nlow << 8) | (packed & 0xffff0000u);
+  if (own) ln.meta[t] = cnt | (nlow << 8) | (packed & 0xffff0000u);
+  // counters, one atomic a warp
+  const uint32_t ntc = __reduce_add_sync(full, packed >> 16);
+  const uint32_t most = __reduce_max_sync(full, cnt);
+  if (lane == 0) {
+    if (ntc) atomicAdd(&ctl->mesh_candidates, ntc);
+    if (most > ctl->max_list_len) atomicMax(&ctl->max_list_len, most);
+  }
 }
 
 __global__ void k_rebuild_end(Ctl* ctl, Params p) {
@@ -612,7 +645,7 @@ k_mirror(Ctl* ctl, Params p, Lists L) {
   }
 }
 
-int64_t list_block_sums_size(int64_t n) { return blocks_for(n, kBuildThreads) + 1; }
+int64_t list_block_sums_size(int64_t n) { return blocks_for(n, kTotalSlots) + 1; }
 
 void launch_mesh_cells(cudaStream_t st, Ctl* ctl, const Params& p, BinBuf bb, MeshDev mesh) {
   const unsigned gcells = (unsigned)std::min<int64_t>(blocks_for(p.ncells, kThreads), 152 * 16);
@@ -627,6 +660,33 @@ void launch_mesh_cells(cudaStream_t st, Ctl* ctl, const Params& p, BinBuf bb, Me
   k_tri_cell_sort<<<152 * 8, 32 * kSortWarps, 0, st>>>(p, bb);
 }
 
+namespace {
+
+template <typename Hist, int G>
+void launch_list_build(cudaStream_t st, Ctl* ctl, const Params& p, Lists L, BinBuf bb,
+                       MeshDev mesh) {
+  k_list_build<Hist, G><<<blocks_for((int64_t)p.n * G, kBuildThreads), kBuildThreads, 0, st>>>(
+      ctl, p, bb, L, mesh);
+}
+
+template <typename Hist>
+void launch_lists(cudaStream_t st, Ctl* ctl, const Params& p, Lists L, BinBuf bb, MeshDev mesh) {
+  if (p.n <= 100000)
+    launch_list_build<Hist, 4>(st, ctl, p, L, bb, mesh);
+  else if (p.n <= 400000)
+    launch_list_build<Hist, 2>(st, ctl, p, L, bb, mesh);
+  else
+    launch_list_build<Hist, 1>(st, ctl, p, L, bb, mesh);
+  const unsigned nbl = blocks_for(p.n, kTotalSlots);
+  k_list_offsets<<<1, kOffsetThreads, 0, st>>>(ctl, p, bb, L, (int)nbl);
+  if (p.n <= 100000)
+    k_list_compact<Hist, 8><<<nbl, 4 * kTotalSlots, 0, st>>>(ctl, p, bb, L);
+  else
+    k_list_compact<Hist, 32><<<nbl, kTotalSlots, 0, st>>>(ctl, p, bb, L);
+}
+
+}  // namespace
+
 void launch_rebuild(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L,
                     BinBuf bb, MeshDev mesh) {
   const unsigned nb = blocks_for(p.n, kThreads);
@@ -638,17 +698,11 @@ void launch_rebuild(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Li
     k_permute<F8><<<nb, kThreads, 0, st>>>(ctl, p, bb, sb, L);
   else
     k_permute<D4><<<nb, kThreads, 0, st>>>(ctl, p, bb, sb, L);
-  const unsigned nbl = blocks_for(p.n, kBuildThreads);
   if (p.hist32)
-    k_list_build<HistM><<<nbl, kBuildThreads, 0, st>>>(ctl, p, bb, L, mesh);
+    launch_lists<HistM>(st, ctl, p, L, bb, mesh);
   else
-    k_list_build<HistD><<<nbl, kBuildThreads, 0, st>>>(ctl, p, bb, L, mesh);
-  k_list_offsets<<<1, kOffsetThreads, 0, st>>>(ctl, p, bb, L, (int)nbl);
-  if (p.hist32)
-    k_list_compact<HistM><<<nbl, 32 * kCompactWarps, 0, st>>>(ctl, p, bb, L);
-  else
-    k_list_compact<HistD><<<nbl, 32 * kCompactWarps, 0, st>>>(ctl, p, bb, L);
-  if (p.pair_res) k_mirror<<<nbl, kBuildThreads, 0, st>>>(ctl, p, L);
+    launch_lists<HistD>(st, ctl, p, L, bb, mesh);
+  if (p.pair_res) k_mirror<<<blocks_for(p.n, 128), 128, 0, st>>>(ctl, p, L);
   k_rebuild_end<<<1, 1, 0, st>>>(ctl, p);
 }
 
