@@ -297,7 +297,7 @@ void dem_scene_destroy(dem_scene* s);
  * come from params (precision and list fields are ignored).
  *
  * Memory: nothing is allocated.  Scratch is one fixed device array inside the
- * library (about 3.5 MB, kept by every device that loads the library until
+ * library (about 7.6 MB, kept by every device that loads the library until
  * the process exits).  Limits: n <= 131072 particles and at most 262144 grid
  * cells; larger requests return DEM_ERR_INVALID without launching anything.
  * More than 64 touching partners of one particle return DEM_ERR_CAPACITY.

@@ -64,6 +64,17 @@ __device__ __forceinline__ V3<T> spring_vec(V3<T>& u, V3<T> n, V3<T> vm, T k, T 
   return f;
 }
 
+// spring_vec of a spring at zero (a contact's first step), without the
+// projection of a zero vector: the same force, bit for bit (-k u is -0, so
+// -k u - c v is -(c v)).  The spring after the step is not formed.
+template <typename T>
+__device__ __forceinline__ V3<T> spring_vec_new(V3<T> vm, T c, T mu, T fn) {
+  const V3<T> f = mk(-(c * vm.x), -(c * vm.y), -(c * vm.z));
+  const T flen = vnorm(f);
+  const T lim = mu * fn;
+  return flen <= lim ? f : (lim / flen) * f;
+}
+
 template <typename T>
 __device__ __forceinline__ T spring_scalar(T& u, T vm, T k, T c, T mu, T fn, T dt) {
   T f = -k * u - c * vm;
@@ -82,8 +93,9 @@ __device__ __forceinline__ T spring_scalar(T& u, T vm, T k, T c, T mu, T fn, T d
 // of the contact velocity; om = w_i - w_j (wall: w_i - Omega).  reff is the
 // rolling radius (1/r_i + 1/r_j)^-1 (wall: r_i); rj is unused for walls.  The
 // callers form the differences so each precision can do it without
-// cancellation.
-template <typename T>
+// cancellation.  New: the springs are at zero (a contact's first step) and are
+// not updated.
+template <typename T, bool New = false>
 __device__ __forceinline__ LawOut<T> contact_law(const LawConst<T>& c, V3<T> n, T delta, T Rs,
                                                  T ms, T ri, T rj, T reff, V3<T> dv, V3<T> rw,
                                                  V3<T> om, V3<T>& us, V3<T>& ur, T& ut) {
@@ -105,8 +117,14 @@ __device__ __forceinline__ LawOut<T> contact_law(const LawConst<T>& c, V3<T> n, 
   const T kd = kn * delta;
   const V3<T> fn = mk(kd * n.x - cn * vn.x, kd * n.y - cn * vn.y, kd * n.z - cn * vn.z);
   const T fnm = vnorm(fn);
-  const V3<T> fs = spring_vec(us, n, vs, ks, cs, c.mu_s, fnm, c.dt);
-  const V3<T> fr = spring_vec(ur, n, vr, kn, cn, c.mu_r, fnm, c.dt);
+  V3<T> fs, fr;
+  if constexpr (New) {
+    fs = spring_vec_new(vs, cs, c.mu_s, fnm);
+    fr = spring_vec_new(vr, cn, c.mu_r, fnm);
+  } else {
+    fs = spring_vec(us, n, vs, ks, cs, c.mu_s, fnm, c.dt);
+    fr = spring_vec(ur, n, vr, kn, cn, c.mu_r, fnm, c.dt);
+  }
   const T ft = spring_scalar(ut, vt, ks, cs, c.mu_t, fnm, c.dt);
   const V3<T> fsxn = cross(fs, n);
   const V3<T> tr = Rs * cross(n, fr);
