@@ -120,6 +120,40 @@ int mpnn_segment_sum_perm(int64_t n, int64_t npad, int32_t W, const int64_t* off
 /* ReLU backward: G[i] = 0 where Y[i] <= 0 (fp32, n values). */
 int mpnn_relu_backward(int64_t n, const float* Y, float* G, void* stream);
 
+/* The layers of the network of width 128 (surrogate.py) with their gathers,
+ * concatenations, residuals and sums inside, bitwise equal to the calls above
+ * in sequence.  npad is a multiple of 64, every pointer 16-byte aligned.
+ * Weights are the transposed bf16 copies Wt[outputs][inputs].
+ *
+ * Encode: h = relu(nf Wn) (nf [npad][16]), hb = bf16(h), and p1 [npad][128] =
+ * hb times the first 128 input rows (the receiver's) of the next round's
+ * message layer Wm_next [128][400]. */
+int mpnn_encode_nodes(int64_t n, int64_t npad, const uint16_t* nf, const uint16_t* Wn,
+                      const uint16_t* Wm_next, float* h, uint16_t* hb, float* p1, void* stream);
+
+/* Edge states: eb [E][128] = bf16(relu(ef We)) (ef [E][16]). */
+int mpnn_encode_edges(int64_t E, const uint16_t* ef, const uint16_t* We, uint16_t* eb,
+                      void* stream);
+
+/* One round's messages, relu([h_dst, h_nbr, e, 1] Wm), summed over the edges
+ * each node receives, ascending: Mb [npad][128] bf16 (rows 0 .. n-1 written;
+ * NaN if a bounded wait inside the kernel ran out).  eb: the edge states; p1:
+ * from the node call before.  Optional mask [E][4]: the bits of the message
+ * components > 0 (component c: word c / 32, bit c % 32). */
+int mpnn_message_sums(int64_t n, int64_t E, const int64_t* off, const int32_t* nbr,
+                      const int32_t* dst, const uint16_t* hb, const uint16_t* eb,
+                      const uint16_t* Wm, const float* p1, uint16_t* Mb, uint32_t* mask,
+                      void* stream);
+
+/* Node update: h += relu([hb_in, Mb, 1] Wu) (rows past n: plus nothing), hb =
+ * bf16(h) (may be hb_in), then out = p1 for the next round (W_next the message
+ * layer [128][400], out [npad][128]) or, with decode nonzero, the outputs
+ * [hb, 1] W_next (W_next [64][144], out [npad][64]).  Optional mask [npad][4]:
+ * the bits of the update components > 0. */
+int mpnn_update_nodes(int64_t n, int64_t npad, const uint16_t* hb_in, const uint16_t* Mb,
+                      const uint16_t* Wu, const uint16_t* W_next, int32_t decode, float* h,
+                      uint16_t* hb, float* out, uint32_t* mask, void* stream);
+
 /* Adam step (bias-corrected, step t >= 1) on n fp32 parameters W with
  * moments m, v and gradient G.  Also writes the bf16 copy Wb (same layout,
  * may be NULL) and, if Wt is not NULL, the transposed bf16 copy of the

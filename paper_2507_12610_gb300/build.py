@@ -19,7 +19,8 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libdem.so")
 
 SOURCES = ["dem_api.cu", "dem_rebuild.cu", "dem_scan.cu", "dem_step.cu", "dem_step_fp64.cu",
-           "dem_noalloc.cu", "dem_spawn.cu", "dem_export.cu", "mpnn.cu", "dem_probe.cu"]
+           "dem_noalloc.cu", "dem_spawn.cu", "dem_export.cu", "mpnn.cu", "mpnn_layers.cu",
+           "dem_probe.cu"]
 # the FP64 step is the precision reference: no multiply-add contraction
 # the mixed step uses approximate FP32 division and square root (about 1 ulp);
 # its compensated sums use neither
@@ -54,7 +55,7 @@ def build(verbose: bool = False, ptxas_info: bool = False, force: bool = False,
     """Compile (if stale) and link libdem.so; extra_flags go to every nvcc call."""
     os.makedirs(build_dir, exist_ok=True)
     headers = [os.path.join(csrc, f) for f in os.listdir(csrc) if f.endswith(".cuh")]
-    headers.append(os.path.join(INCLUDE, "dem.h"))
+    headers += [os.path.join(INCLUDE, h) for h in ("dem.h", "mpnn.h")]
     nv = nvcc()
     jobs = []
     objs = []

@@ -30,7 +30,8 @@ EXPORTS = ("mpnn_gemm", "mpnn_gemm_split", "mpnn_transpose_bf16", "mpnn_to_bf16"
            "mpnn_graph", "mpnn_graph_cells", "mpnn_reverse_edges", "mpnn_features", "mpnn_gather_edges",
            "mpnn_concat_rows", "mpnn_residual", "mpnn_gather_rows", "mpnn_segment_sum",
            "mpnn_segment_sum_cols", "mpnn_segment_sum_perm", "mpnn_relu_backward",
-           "mpnn_adam", "mpnn_mse")
+           "mpnn_adam", "mpnn_mse", "mpnn_encode_nodes", "mpnn_encode_edges",
+           "mpnn_message_sums", "mpnn_update_nodes")
 
 H = 128          # hidden width
 ROUNDS = 3       # message-passing rounds
@@ -175,6 +176,9 @@ class MPNN:
 
     # ---- forward -------------------------------------------------------------
     def forward(self, g: Graph, keep=True):
+        if not keep:
+            self.state = None
+            return self._forward_fused(g)
         torch = self.torch
         dev = torch.device("cuda")
         n, npad, E, Epad = g.n, g.npad, g.E, g.Epad
@@ -210,6 +214,30 @@ class MPNN:
         y = gemm(npad, 64, H + 16, Xd, "dec", False)
         st["Xd"] = Xd
         self.state = st if keep else None
+        return y
+
+    def _forward_fused(self, g: Graph):
+        """forward() by the fused layers, keeping nothing for a backward pass:
+        the same values bit for bit."""
+        torch = self.torch
+        dev = torch.device("cuda")
+        f32, b16 = torch.float32, torch.int16
+        h = torch.empty((g.npad, H), dtype=f32, device=dev)
+        hb = torch.empty((g.npad, H), dtype=b16, device=dev)
+        p1 = torch.empty((g.npad, H), dtype=f32, device=dev)
+        Mb = torch.empty((g.npad, H), dtype=b16, device=dev)
+        eb = torch.empty((g.Epad, H), dtype=b16, device=dev)
+        y = torch.empty((g.npad, 64), dtype=f32, device=dev)
+        _call("mpnn_encode_edges", g.E, g.ef, self.Wt["edge"], eb, None)
+        _call("mpnn_encode_nodes", g.n, g.npad, g.nf, self.Wt["node"], self.Wt["msg0"], h, hb, p1,
+              None)
+        for r in range(ROUNDS):
+            last = r == ROUNDS - 1
+            _call("mpnn_message_sums", g.n, g.E, g.off, g.nbr, g.dst, hb, eb,
+                  self.Wt[f"msg{r}"], p1, Mb, None, None)
+            _call("mpnn_update_nodes", g.n, g.npad, hb, Mb, self.Wt[f"upd{r}"],
+                  self.Wt["dec" if last else f"msg{r + 1}"], _i32(last), h, hb,
+                  y if last else p1, None, None)
         return y
 
     # ---- backward ------------------------------------------------------------
