@@ -154,6 +154,47 @@ int mpnn_update_nodes(int64_t n, int64_t npad, const uint16_t* hb_in, const uint
                       const uint16_t* Wu, const uint16_t* W_next, int32_t decode, float* h,
                       uint16_t* hb, float* out, uint32_t* mask, void* stream);
 
+/* Backward of the fused layers.  zb is the bf16 gradient of a layer's output
+ * before its relu (zero where the relu cut it off); W the bf16 copies
+ * W[inputs][outputs]; gradients of the states add up in the order of the calls
+ * above in sequence (the same bits).  Pointers are 16-byte aligned.
+ *
+ * Decoder: dh [npad][128] = dyb [npad][64] times Wdec^T, and zb [npad][128] of
+ * the last update layer (mask: its bits). */
+int mpnn_grad_decode(int64_t npad, const uint16_t* dyb, const uint16_t* Wdec,
+                     const uint32_t* mask, float* dh, uint16_t* zb, void* stream);
+
+/* Update layer: dh += the state's part of zb Wu^T; dMb = the message sums' part. */
+int mpnn_grad_update(int64_t npad, const uint16_t* zb, const uint16_t* Wu, float* dh,
+                     uint16_t* dMb, void* stream);
+
+/* Message layer: zm [E][128], the edge's gradient, is dMb[dst] where its mask bits
+ * are set and 0 elsewhere; dX
+ * [E][256] = the receiver's and sender's parts of it times Wm^T; de [E][128] the
+ * edge state's, starting at 0 with `first`; with `last` it is not stored, and zeb
+ * [E][128] = bf16(de) where eb > 0. */
+int mpnn_grad_messages(int64_t E, const int32_t* dst, const uint16_t* dMb, const uint32_t* mask,
+                       const uint16_t* Wm, const uint16_t* eb, int32_t first, int32_t last,
+                       uint16_t* zm, float* dX, float* de, uint16_t* zeb, void* stream);
+
+/* Nodes: dh = (dh + the sum of dX[e][0..128) over the edges received) + the sum of
+ * dX[perm][128..256) over those sent; zb = bf16(dh) where the bits of mask are set
+ * or, with mask NULL, where hb > 0. */
+int mpnn_grad_nodes(int64_t n, int64_t npad, const int64_t* off, const int32_t* perm,
+                    const float* dX, const uint32_t* mask, const uint16_t* hb, float* dh,
+                    uint16_t* zb, void* stream);
+
+/* Weights: G [kp][N] = [X0[idx0], X1[idx1], X2, 1]^T dZ over `rows` rows, of the
+ * first `segments` (1 to 3) inputs of width 128 each; idx NULL: the row itself.
+ * segments 0: X0 of width 16 alone, no constant.  N = 128 (one segment: or 64).
+ * Rows of G past the inputs are zero.  The bits are those of mpnn_gemm_split over K
+ * >= rows rows (zeros after `rows`, K % 16 == 0) in `splits` parts; work
+ * [splits][kp][N], caller-owned. */
+int mpnn_grad_weights(int64_t rows, int64_t K, int32_t segments, const uint16_t* X0,
+                      const int32_t* idx0, const uint16_t* X1, const int32_t* idx1,
+                      const uint16_t* X2, const uint16_t* dZ, int32_t N, int32_t kp,
+                      int32_t splits, float* work, float* G, void* stream);
+
 /* Adam step (bias-corrected, step t >= 1) on n fp32 parameters W with
  * moments m, v and gradient G.  Also writes the bf16 copy Wb (same layout,
  * may be NULL) and, if Wt is not NULL, the transposed bf16 copy of the
@@ -162,7 +203,7 @@ int mpnn_adam(int64_t n, float* W, float* m, float* v, const float* G, float lr,
               float beta2, float eps, int64_t t, uint16_t* Wb, uint16_t* Wt, int32_t rows,
               int32_t cols, int32_t kin, void* stream);
 
-/* out[0] = sum of (a - b)^2 over n values (one block, fixed order), and
+/* out[0] = sum of (a - b)^2 over n values (in a fixed order), and
  * G = 2 (a - b) * scale. */
 int mpnn_mse(int64_t n, const float* a, const float* b, float scale, float* G, float* out,
              void* stream);

@@ -136,7 +136,8 @@ struct MessageArgs {
 
 // One block an SM owns a range of nodes (of about the same cost for every block:
 // the start and sum warps work by node, so a node counts as kNodeCost edges; with
-// 1 the blocks of a bed's loose top took twice as long as the others) and takes their edges 128 at a time: two tiles of
+// 1 the blocks of a bed's loose top took twice as long as the others) and takes
+// their edges 128 at a time: two tiles of
 // operands in shared memory, four of accumulators in TMEM.  Products are taken
 // transposed: TMEM lane c holds message component c of the tile's edges
 // (columns), so that one thread has a component of consecutive edges and sums a

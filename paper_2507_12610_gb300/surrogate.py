@@ -31,7 +31,8 @@ EXPORTS = ("mpnn_gemm", "mpnn_gemm_split", "mpnn_transpose_bf16", "mpnn_to_bf16"
            "mpnn_concat_rows", "mpnn_residual", "mpnn_gather_rows", "mpnn_segment_sum",
            "mpnn_segment_sum_cols", "mpnn_segment_sum_perm", "mpnn_relu_backward",
            "mpnn_adam", "mpnn_mse", "mpnn_encode_nodes", "mpnn_encode_edges",
-           "mpnn_message_sums", "mpnn_update_nodes")
+           "mpnn_message_sums", "mpnn_update_nodes", "mpnn_grad_decode", "mpnn_grad_update",
+           "mpnn_grad_messages", "mpnn_grad_nodes", "mpnn_grad_weights")
 
 H = 128          # hidden width
 ROUNDS = 3       # message-passing rounds
@@ -176,144 +177,78 @@ class MPNN:
 
     # ---- forward -------------------------------------------------------------
     def forward(self, g: Graph, keep=True):
-        if not keep:
-            self.state = None
-            return self._forward_fused(g)
+        """The outputs [npad][64] (fp32); keep: also the states and relu masks that
+        backward() needs."""
         torch = self.torch
-        dev = torch.device("cuda")
-        n, npad, E, Epad = g.n, g.npad, g.E, g.Epad
-        st = {}
-        z = self.zero_bias
+        f32, b16, i32 = torch.float32, torch.int16, torch.int32
+        n, npad, E = g.n, g.npad, g.E
 
-        def gemm(M, N, K, A, name, relu, C=None, Cb=None):
-            C = torch.empty((M, N), dtype=torch.float32, device=dev) if C is None else C
-            _call("mpnn_gemm", M, N, K, A, self.Wt[name], C, Cb, z, _i32(2 if relu else 0),
-                  _i32(0), None)
-            return C
+        def new(rows, cols, dtype):
+            return torch.empty((rows, cols), dtype=dtype, device=torch.device("cuda"))
 
-        hb = torch.empty((npad, H), dtype=torch.int16, device=dev)
-        h = gemm(npad, H, 16, g.nf, "node", True, Cb=hb)
-        st["h0"] = h.clone()
-        eb = torch.empty((Epad, H), dtype=torch.int16, device=dev)
-        e = gemm(Epad, H, 16, g.ef, "edge", True, Cb=eb)
-        st["e"] = e
-        for r in range(ROUNDS):
-            Xm = torch.empty((Epad, 3 * H + 16), dtype=torch.int16, device=dev)
-            _call("mpnn_gather_edges", E, Epad, _i32(H), _i32(H), g.dst, g.nbr, hb, eb, Xm, None)
-            m = gemm(Epad, H, 3 * H + 16, Xm, f"msg{r}", True)
-            Mi = torch.empty((npad, H), dtype=torch.float32, device=dev)
-            _call("mpnn_segment_sum", n, npad, _i32(H), g.off, m, Mi, None)
-            Xu = torch.empty((npad, 2 * H + 16), dtype=torch.int16, device=dev)
-            _call("mpnn_concat_rows", n, npad, _i32(H), _i32(H), hb, Mi, Xu, None)
-            u = gemm(npad, H, 2 * H + 16, Xu, f"upd{r}", True)
-            _call("mpnn_residual", npad * H, h, u, hb, None)
-            if keep:
-                st[f"Xm{r}"], st[f"m{r}"], st[f"Xu{r}"], st[f"u{r}"] = Xm, m, Xu, u
-        Xd = torch.empty((npad, H + 16), dtype=torch.int16, device=dev)
-        _call("mpnn_concat_rows", n, npad, _i32(H), _i32(0), hb, None, Xd, None)
-        y = gemm(npad, 64, H + 16, Xd, "dec", False)
-        st["Xd"] = Xd
-        self.state = st if keep else None
-        return y
-
-    def _forward_fused(self, g: Graph):
-        """forward() by the fused layers, keeping nothing for a backward pass:
-        the same values bit for bit."""
-        torch = self.torch
-        dev = torch.device("cuda")
-        f32, b16 = torch.float32, torch.int16
-        h = torch.empty((g.npad, H), dtype=f32, device=dev)
-        hb = torch.empty((g.npad, H), dtype=b16, device=dev)
-        p1 = torch.empty((g.npad, H), dtype=f32, device=dev)
-        Mb = torch.empty((g.npad, H), dtype=b16, device=dev)
-        eb = torch.empty((g.Epad, H), dtype=b16, device=dev)
-        y = torch.empty((g.npad, 64), dtype=f32, device=dev)
-        _call("mpnn_encode_edges", g.E, g.ef, self.Wt["edge"], eb, None)
-        _call("mpnn_encode_nodes", g.n, g.npad, g.nf, self.Wt["node"], self.Wt["msg0"], h, hb, p1,
-              None)
+        self.state = None
+        h, hb = new(npad, H, f32), new(npad, H, b16)
+        p1, y = new(npad, H, f32), new(npad, 64, f32)
+        Mb, eb = new(npad, H, b16), new(g.Epad, H, b16)
+        st = dict(hb=[hb], Mb=[], m=[], u=[], eb=eb)
+        _call("mpnn_encode_edges", E, g.ef, self.Wt["edge"], eb, None)
+        _call("mpnn_encode_nodes", n, npad, g.nf, self.Wt["node"], self.Wt["msg0"], h, hb, p1, None)
+        m = u = None
         for r in range(ROUNDS):
             last = r == ROUNDS - 1
-            _call("mpnn_message_sums", g.n, g.E, g.off, g.nbr, g.dst, hb, eb,
-                  self.Wt[f"msg{r}"], p1, Mb, None, None)
-            _call("mpnn_update_nodes", g.n, g.npad, hb, Mb, self.Wt[f"upd{r}"],
+            hb_in = hb
+            if keep:
+                hb, Mb = new(npad, H, b16), new(npad, H, b16)
+                m, u = new(g.Epad, H // 32, i32), new(npad, H // 32, i32)
+                for key, t in (("hb", hb), ("Mb", Mb), ("m", m), ("u", u)):
+                    st[key].append(t)
+            _call("mpnn_message_sums", n, E, g.off, g.nbr, g.dst, hb_in, eb, self.Wt[f"msg{r}"],
+                  p1, Mb, m, None)
+            _call("mpnn_update_nodes", n, npad, hb_in, Mb, self.Wt[f"upd{r}"],
                   self.Wt["dec" if last else f"msg{r + 1}"], _i32(last), h, hb,
-                  y if last else p1, None, None)
+                  y if last else p1, u, None)
+        if keep:
+            self.state = st
         return y
 
     # ---- backward ------------------------------------------------------------
-    def _wgrad(self, name, X, rows, dZ):
-        """G[name] = X^T dZ with X (bf16 [rows][kin]) and dZ (fp32 [rows][N])."""
-        torch = self.torch
-        dev = torch.device("cuda")
-        kin, nout = LAYERS[name]
-        kp = pad64(kin)
-        XT = torch.zeros((kp, rows), dtype=torch.int16, device=dev)
-        _call("mpnn_transpose_bf16", kin, rows, X, XT, None)
-        dZb = torch.empty((rows, nout), dtype=torch.int16, device=dev)
-        _call("mpnn_to_bf16", rows * nout, dZ, dZb, None)
-        dZT = torch.empty((nout, rows), dtype=torch.int16, device=dev)
-        _call("mpnn_transpose_bf16", nout, rows, dZb, dZT, None)
-        splits = max(1, min(64, rows // 4096))
-        work = torch.empty((splits, kp, nout), dtype=torch.float32, device=dev)
-        _call("mpnn_gemm_split", kp, nout, rows, _i32(splits), XT, dZT, self.G[name], _i32(0),
-              work, None)
-        return dZb
-
-    def _dx(self, name, dZb, rows):
-        """dX = dZ W^T: fp32 [rows][pad64(kin)]."""
-        torch = self.torch
-        kin, nout = LAYERS[name]
-        kp = pad64(kin)
-        dX = torch.empty((rows, kp), dtype=torch.float32, device=torch.device("cuda"))
-        _call("mpnn_gemm", rows, kp, nout, dZb, self.Wb[name], dX, None, None, _i32(0), _i32(0),
-              None)
-        return dX
-
     def backward(self, g: Graph, dy):
         torch = self.torch
-        dev = torch.device("cuda")
+        f32, b16 = torch.float32, torch.int16
         st = self.state
-        n, npad, E, Epad = g.n, g.npad, g.E, g.Epad
-        dyb = self._wgrad("dec", st["Xd"], npad, dy)
-        dXd = self._dx("dec", dyb, npad)
-        dh = torch.empty((npad, H), dtype=torch.float32, device=dev)
-        _call("mpnn_segment_sum_cols", npad, npad, _i32(H), dXd.shape[1], _i32(0), g.ident_n,
-              None, dXd, dh, None)
-        de = torch.zeros((Epad, H), dtype=torch.float32, device=dev)
-        tmp_b = torch.empty((max(npad, Epad) * H,), dtype=torch.int16, device=dev)
+        n, npad, E = g.n, g.npad, g.E
+
+        def new(rows, cols, dtype):
+            return torch.empty((rows, cols), dtype=dtype, device=torch.device("cuda"))
+
+        # a weight's gradient is summed in row ranges of about 4,096 (64 at most)
+        splits = {rows: max(1, min(64, rows // 4096)) for rows in (npad, g.Epad)}
+        work = new(max(splits[npad], splits[g.Epad]) * pad64(3 * H + 16), H, f32)
+
+        def weights(name, rows, K, segments, X, idx, dZ):
+            kin, nout = LAYERS[name]
+            X, idx = list(X) + [None] * (3 - len(X)), list(idx) + [None] * (2 - len(idx))
+            _call("mpnn_grad_weights", rows, K, _i32(segments), X[0], idx[0], X[1], idx[1], X[2],
+                  dZ, _i32(nout), _i32(pad64(kin)), _i32(splits[K]), work, self.G[name], None)
+
+        dyb, zb = new(npad, 64, b16), new(npad, H, b16)
+        dh, dMb = new(npad, H, f32), new(npad, H, b16)
+        dX, de = new(g.Epad, 2 * H, f32), new(g.Epad, H, f32)
+        zm, zeb = new(g.Epad, H, b16), new(g.Epad, H, b16)
+        _call("mpnn_to_bf16", npad * 64, dy, dyb, None)
+        weights("dec", n, npad, 1, [st["hb"][ROUNDS]], [], dyb)
+        _call("mpnn_grad_decode", npad, dyb, self.Wb["dec"], st["u"][-1], dh, zb, None)
         for r in reversed(range(ROUNDS)):
-            du = dh.clone()
-            _call("mpnn_relu_backward", npad * H, st[f"u{r}"], du, None)
-            dub = self._wgrad(f"upd{r}", st[f"Xu{r}"], npad, du)
-            dXu = self._dx(f"upd{r}", dub, npad)
-            w = dXu.shape[1]
-            part = torch.empty((npad, H), dtype=torch.float32, device=dev)
-            _call("mpnn_segment_sum_cols", npad, npad, _i32(H), w, _i32(0), g.ident_n, None, dXu,
-                  part, None)
-            _call("mpnn_residual", npad * H, dh, part, tmp_b, None)   # dh += d/dh of [h, M]
-            dM = torch.empty((npad, H), dtype=torch.float32, device=dev)
-            _call("mpnn_segment_sum_cols", npad, npad, _i32(H), w, _i32(H), g.ident_n, None, dXu,
-                  dM, None)
-            dm = torch.empty((Epad, H), dtype=torch.float32, device=dev)
-            _call("mpnn_gather_rows", E, Epad, _i32(H), g.dst, dM, dm, None)
-            _call("mpnn_relu_backward", Epad * H, st[f"m{r}"], dm, None)
-            dmb = self._wgrad(f"msg{r}", st[f"Xm{r}"], Epad, dm)
-            dXm = self._dx(f"msg{r}", dmb, Epad)
-            w = dXm.shape[1]
-            _call("mpnn_segment_sum_cols", n, npad, _i32(H), w, _i32(0), g.off, None, dXm, part,
-                  None)
-            _call("mpnn_residual", npad * H, dh, part, tmp_b, None)   # receivers
-            _call("mpnn_segment_sum_cols", n, npad, _i32(H), w, _i32(H), g.off, g.perm, dXm,
-                  part, None)
-            _call("mpnn_residual", npad * H, dh, part, tmp_b, None)   # senders
-            pe = torch.empty((Epad, H), dtype=torch.float32, device=dev)
-            _call("mpnn_segment_sum_cols", Epad, Epad, _i32(H), w, _i32(2 * H), g.ident_e, None,
-                  dXm, pe, None)
-            _call("mpnn_residual", Epad * H, de, pe, tmp_b, None)     # edge embeddings
-        _call("mpnn_relu_backward", Epad * H, st["e"], de, None)
-        self._wgrad("edge", g.ef, Epad, de)
-        _call("mpnn_relu_backward", npad * H, st["h0"], dh, None)
-        self._wgrad("node", g.nf, npad, dh)
+            hb, m = st["hb"][r], st["m"][r]
+            weights(f"upd{r}", n, npad, 2, [hb, st["Mb"][r]], [], zb)
+            _call("mpnn_grad_update", npad, zb, self.Wb[f"upd{r}"], dh, dMb, None)
+            _call("mpnn_grad_messages", E, g.dst, dMb, m, self.Wb[f"msg{r}"], st["eb"],
+                  _i32(r == ROUNDS - 1), _i32(r == 0), zm, dX, de, zeb, None)
+            weights(f"msg{r}", E, g.Epad, 3, [hb, hb, st["eb"]], [g.dst, g.nbr], zm)
+            _call("mpnn_grad_nodes", n, npad, g.off, g.perm, dX, st["u"][r - 1] if r else None,
+                  None if r else st["hb"][0], dh, zb, None)
+        weights("edge", E, g.Epad, 0, [g.ef], [], zeb)
+        weights("node", n, npad, 0, [g.nf], [], zb)
 
     def loss_and_grad(self, g: Graph, target):
         """MSE over the n x 6 outputs; target fp32 [npad][64] (zeros past 6
