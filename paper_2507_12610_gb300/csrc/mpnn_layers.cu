@@ -150,17 +150,26 @@ struct MessageArgs {
 //                     and the chain over k begins with the receiver's columns, so
 //                     the start is exact and saves 8 of 25 chunks);
 //   one thread        issues the 17 chunks of the senders, edges and constant;
-//   8 sum warps       take the messages from TMEM, relu, and sum them node by node,
-//                     each group of 4 every other tile: a group leaves its tile's
+//   12 sum warps      take the messages from TMEM, relu, and sum them node by node,
+//                     each group of 4 every third tile: a group leaves its tile's
 //                     first node to the end, when the sum of that node's edges in
-//                     the tile before has come from the other group.
+//                     the tile before has come from the group before.  (A sum and
+//                     its place in the ring of kCarry are taken before the ring comes
+//                     round: tile t + 8 starts after tile t + 4 has left its
+//                     accumulators, and the group of t + 4 took t + 1 before it.)
 // The weights stay in shared memory (72 KB).  Measured on a settled bed of 100,000
-// nodes and 1,054,942 edges: 157 us, against 1,230 us for the gather, product and
-// sum kernels it replaces (23,026 edges: 16 us); bound by the start and sum warps'
-// work on runs of about ten edges, then by the L2 reads of both states (52 us of
-// HBM traffic, 20 us of products).
+// nodes and 1,054,942 edges: 125 us, against 1,230 us for the gather, product and
+// sum kernels it replaces (20,000 nodes: 27 us).  Bound by the issue slots (60 %
+// busy) that the start and sum warps take for runs of about ten edges, then by the
+// L2 reads of both states (52 us of HBM traffic, 20 us of products).  With two
+// groups of sum warps 157 us (20,000: 37), with three and two comparisons a column
+// 151; the rest is the search for a block's first node.
 constexpr int kTileE = 128;
-constexpr int kMsgThreads = 21 * 32;
+constexpr int kSumGroups = 3;
+// first warps of the roles (each on a multiple of 4: a warp reaches the 32 TMEM
+// lanes of its number mod 4)
+constexpr int kStartWarp = 4 * kSumGroups, kCopyWarp = kStartWarp + 8, kIssueWarp = kCopyWarp + 4;
+constexpr int kMsgThreads = 32 * (kIssueWarp + 1);
 constexpr uint32_t kPanel = 128 * 128;  // 128 rows of 64 bf16
 constexpr uint32_t kPlain = 128 * 32;   // 128 rows of 16 bf16
 // stages: senders (2 panels), edge states (2 panels)
@@ -177,7 +186,7 @@ struct MsgShared {
   int node[2];
   int failed;
   int2 start[8][65];          // runs of edges of one node, by start warp
-  int2 run[8][kTileE + 2];    // ... by sum warp
+  int2 run[kStartWarp][kTileE + 2];  // ... by sum warp
   float carry[kCarry][128];   // open sum at the end of a tile
 };
 
@@ -268,15 +277,20 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
     *reinterpret_cast<uint4*>(smem + kMsgXc + (k >> 7) * 2048 + 16 * (k & 127)) =
         make_uint4(k < 128 ? 0x3F80u : 0u, 0u, 0u, 0u);
   cp_commit();
-  if (tid < 2) {  // first node whose edges and nodes before it reach the share
-    const int64_t share = (a.E + kNodeCost * a.n) * (int64_t)(blockIdx.x + tid) / gridDim.x;
+  if (warp < 2) {
+    // first node whose edges and nodes before it reach the share; a warp probes 32
+    // nodes at a time (one by one the dependent loads were most of the 8 us before
+    // the first tile)
+    const int64_t share = (a.E + kNodeCost * a.n) * (int64_t)(blockIdx.x + warp) / gridDim.x;
     int64_t lo = 0, hi = a.n;
     while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (a.off[mid] + kNodeCost * mid < share) lo = mid + 1;
-      else hi = mid;
+      const int64_t chunk = (hi - lo + 31) / 32, at = lo + lane * chunk;
+      const bool before = at < hi && a.off[at] + kNodeCost * at < share;
+      const int k = __popc(__ballot_sync(0xffffffffu, before));
+      hi = k < 32 ? min(hi, lo + k * chunk) : hi;
+      lo = k > 0 ? lo + (k - 1) * chunk + 1 : lo;
     }
-    S.node[tid] = (int)(blockIdx.x + tid == gridDim.x ? a.n : lo);
+    if (lane == 0) S.node[warp] = (int)(blockIdx.x + warp == gridDim.x ? a.n : lo);
   }
   if (tid == 64) {
     for (int b = 0; b < 2; ++b) mbar_init(bar(&S.full[b]), 128);
@@ -289,7 +303,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
     S.failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 20) tc_alloc(smem_addr(&S.tmem), 512);
+  if (warp == kIssueWarp) tc_alloc(smem_addr(&S.tmem), 512);
   cp_wait<0>();
   fence_async_smem();
   tc_fence_before();
@@ -301,7 +315,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
   const int ntile = (int)((e_end - e_begin + kTileE - 1) / kTileE);
   volatile int* failed = &S.failed;
 
-  if (warp == 20) {
+  if (warp == kIssueWarp) {
     // ---- issuer
     if (lane == 0) {
       const uint32_t idesc = tc_idesc(128, 128);
@@ -322,9 +336,9 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       }
     }
     __syncwarp();
-  } else if (warp >= 16) {
+  } else if (warp >= kCopyWarp) {
     // ---- producers: warp w copies rows 32 w .. 32 w + 31 of a tile, two a step
-    const int w = warp - 16;
+    const int w = warp - kCopyWarp;
     int next = ntile > 0 ? a.src[min(e_begin + 32 * w + lane, e_end - 1)] : 0;
     for (int t = 0; t < ntile; ++t) {
       const int b = t & 1;
@@ -353,11 +367,11 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
     cp_wait<0>();
     fence_async_smem();
     if (ntile > 0) mbar_arrive(bar(&S.full[(ntile - 1) & 1]));
-  } else if (warp >= 8) {
+  } else if (warp >= kStartWarp) {
     // ---- start warps: thread = component, group = half of the tile's edges
-    const int half = (warp - 8) >> 2, c = tid & 127;
+    const int half = (warp - kStartWarp) >> 2, c = tid & 127;
     const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
-    int2* const run = S.start[warp - 8];
+    int2* const run = S.start[warp - kStartWarp];
     Receivers R;
     if (ntile > 0) R.load(a.dst, e_begin + 64 * half, e_begin, e_end, lane);
     for (int t = 0; t < ntile; ++t) {
@@ -375,7 +389,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       mbar_arrive(bar(&S.ready[d]));
     }
   } else {
-    // ---- sum warps: thread = component, group = tiles of one parity
+    // ---- sum warps: thread = component, group = every third tile
     const int group = warp >> 2, c = tid & 127;
     const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
     int2* const run = S.run[warp];
@@ -389,7 +403,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       }
     };
     if (group < ntile) receivers(e_begin + group * kTileE);
-    for (int t = group; t < ntile; t += 2) {
+    for (int t = group; t < ntile; t += kSumGroups) {
       const int d = t & 3;
       const int64_t t0 = e_begin + (int64_t)t * kTileE;
       // the tile's runs of edges of one node: (edge after the last, receiver); a
@@ -407,7 +421,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       }
       if (lane < 2) run[nrun + lane] = make_int2(m, -1);
       __syncwarp();
-      if (t + 2 < ntile) receivers(t0 + 2 * kTileE);
+      if (t + kSumGroups < ntile) receivers(t0 + kSumGroups * kTileE);
       const bool ok = mbar_wait(bar(&S.mdone[d]), (t >> 2) & 1, failed);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
@@ -420,16 +434,18 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
           const int from = min(pos, kTileE - 16);
           uint32_t v[16];
           tc_ld16(v, acc + (uint32_t)from);
-          const int skip = pos - from, stop = end - from;
+          // the columns that count, as bits: one test sets seven predicates, where two
+          // comparisons a column took half of the sum warps' instructions
+          const int stop = min(end - from, 16);
+          const uint32_t in = ((1u << stop) - 1u) & ~((1u << (pos - from)) - 1u);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            // (s is never -0, so the sign of a zero term does not matter)
-            const bool in = j >= skip && j < stop;
-            const float x = in ? fmaxf(__uint_as_float(v[j]), 0.f) : 0.f;
-            s += x;
+            const float x = fmaxf(__uint_as_float(v[j]), 0.f);
+            if (in >> j & 1u) s += x;
             if (Keep) {
               const uint32_t bits = __ballot_sync(0xffffffffu, x > 0.f);
-              if (lane == j && in) a.mask[(t0 + from + j) * 4 + (warp & 3)] = bits;
+              if (lane == j && (in >> j & 1u))
+                a.mask[(t0 + from + j) * 4 + (warp & 3)] = bits;
             }
           }
           pos = from + 16;
@@ -472,7 +488,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       }
     }
     // nodes without edges
-    for (int i = i0 + tid; i < i1; i += 256)
+    for (int i = i0 + tid; i < i1; i += 128 * kSumGroups)
       if (a.off[i] == a.off[i + 1])
         for (int k = 0; k < kH / 8; ++k)
           reinterpret_cast<uint4*>(a.Mb + (int64_t)i * kH)[k] = make_uint4(0u, 0u, 0u, 0u);
@@ -483,7 +499,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
     for (int64_t k = tid; k < (int64_t)(i1 - i0) * kH; k += kMsgThreads)
       a.Mb[(int64_t)i0 * kH + k] = 0x7FC0u;
   }
-  if (warp == 20) {
+  if (warp == kIssueWarp) {
     tc_fence_after();
     tc_dealloc(tmem, 512);
   }
