@@ -549,7 +549,8 @@ k_scan_tiles(int64_t n, int64_t* cnt, int64_t* __restrict__ off) {
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_add(int64_t n, const int64_t* __restrict__ cnt, int64_t* __restrict__ off) {
+k_scan_add(int64_t n, const int64_t* __restrict__ cnt, int64_t* __restrict__ off,
+           int64_t* __restrict__ total) {
   __shared__ int64_t warp_s[kScanThreads / 32];
   const int64_t b = blockIdx.x, base = b * kScanTile;
   int64_t before = 0;
@@ -557,13 +558,17 @@ k_scan_add(int64_t n, const int64_t* __restrict__ cnt, int64_t* __restrict__ off
   before = block_sum(before, warp_s);
   for (int k = threadIdx.x; k < kScanTile; k += kScanThreads)
     if (base + k < n) off[base + k] += before;
-  if (base + kScanTile >= n && threadIdx.x == 0) off[n] = before + cnt[base];
+  if (base + kScanTile >= n && threadIdx.x == 0) {
+    off[n] = before + cnt[base];
+    if (total) *total = off[n];
+  }
 }
 
-void scan_counts(int64_t n, int64_t* cnt, int64_t* off, cudaStream_t st) {
+void scan_counts(int64_t n, int64_t* cnt, int64_t* off, cudaStream_t st,
+                 int64_t* total = nullptr) {
   const unsigned nb = (unsigned)((n + kScanTile - 1) / kScanTile);
   k_scan_tiles<<<nb, kScanThreads, 0, st>>>(n, cnt, off);
-  k_scan_add<<<nb, kScanThreads, 0, st>>>(n, cnt, off);
+  k_scan_add<<<nb, kScanThreads, 0, st>>>(n, cnt, off, total);
 }
 
 // perm[k] for k in node j's row (edges received by j, neighbour i = nbr[k]):
@@ -831,27 +836,28 @@ int mpnn_graph_cells(int64_t n, const float* x, float cutoff, int64_t max_cells,
   int64_t* cstart = work + (max_cells + 1);
   int64_t* keyloc = cstart + (max_cells + 1);
   int32_t* order = reinterpret_cast<int32_t*>(keyloc + n);
-  unsigned int* maxdeg = reinterpret_cast<unsigned int*>(order + n);
-  if (cudaMemsetAsync(ccount, 0, sizeof(int64_t) * (ncells + 1), st) != cudaSuccess ||
-      cudaMemsetAsync(maxdeg, 0, sizeof(unsigned int), st) != cudaSuccess)
+  if (cudaMemsetAsync(ccount, 0, sizeof(int64_t) * (ncells + 1), st) != cudaSuccess)
     return DEM_ERR_CUDA;
   const unsigned nb = grid_for(n, 256);
   k_cells_count<<<nb, 256, 0, st>>>(n, x, g, ccount, keyloc);
   scan_counts(ncells, reinterpret_cast<int64_t*>(ccount), cstart, st);
   k_cells_scatter<<<nb, 256, 0, st>>>(n, keyloc, cstart, order);
+  // the counts are done with: their first words take the edge count and the largest
+  // degree, read back by one copy
+  unsigned int* maxdeg = reinterpret_cast<unsigned int*>(work + 1);
+  if (cudaMemsetAsync(work, 0, 2 * sizeof(int64_t), st) != cudaSuccess) return DEM_ERR_CUDA;
   const float c2 = cutoff * cutoff;
   const unsigned nbg = (unsigned)((n * kNodeLanes + kGraphThreads - 1) / kGraphThreads);
   k_graph_cells<<<nbg, kGraphThreads, 0, st>>>(n, x, g, c2, 0, cstart, order, cnt, nullptr, nullptr,
                                        maxdeg);
-  scan_counts(n, cnt, off, st);
-  int64_t E = 0;
-  unsigned int md = 0;
-  if (cudaMemcpyAsync(&E, off + n, sizeof E, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaMemcpyAsync(&md, maxdeg, sizeof md, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  scan_counts(n, cnt, off, st, work);
+  int64_t read[2] = {0, 0};
+  if (cudaMemcpyAsync(read, work, sizeof read, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return DEM_ERR_CUDA;
+  const int64_t E = read[0], md = read[1];
   if (n_edges_host) *n_edges_host = E;
-  if (md > (unsigned)kMaxDegree) return DEM_ERR_CAPACITY;
+  if (md > kMaxDegree) return DEM_ERR_CAPACITY;
   if (E > max_edges || !nbr || !dst) return E > max_edges ? DEM_ERR_CAPACITY : DEM_ERR_INVALID;
   k_graph_cells<<<nbg, kGraphThreads, 0, st>>>(n, x, g, c2, 1, cstart, order, off, nbr, dst, maxdeg);
   return launch_status();

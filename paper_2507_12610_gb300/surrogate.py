@@ -57,32 +57,55 @@ def load():
         lib = _dem.load()
         for name in EXPORTS:
             getattr(lib, name).restype = ctypes.c_int
+        import torch
+        _CONVERT[torch.Tensor] = lambda t: ctypes.c_void_p(t.data_ptr())
         _lib = lib
     return _lib
 
 
+# C arguments by Python type (other types: C values as they are, or tensors)
+_CONVERT = {int: ctypes.c_int64, float: ctypes.c_float, bool: ctypes.c_int32,
+            type(None): lambda _: ctypes.c_void_p(0), ctypes.c_int32: lambda v: v}
+
+
+def _convert(a):
+    if isinstance(a, (ctypes._SimpleCData, ctypes._Pointer)):
+        return a
+    for t in (float, bool, int):  # and types derived from them
+        if isinstance(a, t):
+            return _CONVERT[t](a)
+    return ctypes.c_void_p(a.data_ptr())
+
+
 def _call(name, *args):
-    conv = []
-    for a in args:
-        if isinstance(a, float):
-            conv.append(ctypes.c_float(a))
-        elif isinstance(a, bool):
-            conv.append(ctypes.c_int32(int(a)))
-        elif isinstance(a, int):
-            conv.append(ctypes.c_int64(a))
-        elif a is None:
-            conv.append(ctypes.c_void_p(0))
-        elif isinstance(a, (ctypes._SimpleCData, ctypes._Pointer)):
-            conv.append(a)
-        else:  # a torch tensor
-            conv.append(ctypes.c_void_p(a.data_ptr()))
-    rc = getattr(load(), name)(*conv)
+    get = _CONVERT.get
+    lib = _lib or load()
+    rc = getattr(lib, name)(*[get(type(a), _convert)(a) for a in args])
     if rc != 0:
         raise _dem.DemError(rc, name)
 
 
 def _i32(v):
     return ctypes.c_int32(int(v))
+
+
+def _upload(arrays, dev):
+    """Float32 copies of host arrays on the device, each from a 16-byte boundary, by
+    one transfer (four transfers and numpy's one-thread conversion were 0.4 ms of a
+    100,000-sphere stride)."""
+    import torch
+    arrays = [np.asarray(a) for a in arrays]
+    start = np.cumsum([0] + [(a.size + 3) // 4 * 4 for a in arrays]).tolist()
+    host = torch.empty(start[-1], dtype=torch.float32)
+    for a, k in zip(arrays, start):
+        part = host[k:k + a.size].view(a.shape)
+        if a.dtype in (np.float64, np.float32) and a.flags.writeable and a.dtype.isnative \
+                and min(a.strides, default=0) >= 0:
+            part.copy_(torch.from_numpy(a))
+        else:
+            part.numpy()[...] = a
+    buf = host.to(dev)
+    return [buf[k:k + a.size].view(a.shape) for a, k in zip(arrays, start)]
 
 
 class Graph:
@@ -96,8 +119,7 @@ class Graph:
         dev = torch.device("cuda")
         n = int(R.shape[0])
         self.n, self.npad = n, pad64(n)
-        f32 = lambda a: torch.as_tensor(np.ascontiguousarray(a, dtype=np.float32), device=dev)
-        self.x, self.v, self.w, self.R = f32(x), f32(v), f32(w), f32(R)
+        self.x, self.v, self.w, self.R = _upload((x, v, w, R), dev)
         cnt = torch.empty(n, dtype=torch.int64, device=dev)
         self.off = torch.empty(n + 1, dtype=torch.int64, device=dev)
         ne = ctypes.c_int64(0)
@@ -121,9 +143,6 @@ class Graph:
         self.ef = torch.empty(self.Epad * 16, dtype=torch.int16, device=dev)
         _call("mpnn_features", n, self.npad, self.E, self.Epad, self.dst, self.nbr, self.x,
               self.v, self.w, self.R, float(vs), float(Rs), self.nf, self.ef, None)
-        # identity offsets: a one-row "segment" per node / per edge (column copies)
-        self.ident_n = torch.arange(self.npad + 1, dtype=torch.int64, device=dev)
-        self.ident_e = torch.arange(self.Epad + 1, dtype=torch.int64, device=dev)
 
     def edges_host(self):
         off = self.off.cpu().numpy()
