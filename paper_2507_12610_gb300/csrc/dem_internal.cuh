@@ -160,8 +160,8 @@ struct ListBuf {
                     // the partner's entry for the same pair (one evaluation per pair)
   uint8_t* back;    // [offs[n]] for an entry whose partner has the higher caller index,
                     // the index of this particle in the partner's list
-  D4* inv;          // [n] DEM_FP64 only (else null): 1/R, 1/m, 1/I of the particle in
-                    // each slot, the divisions of the law done once per rebuild
+  D4* inv;          // [n] DEM_FP64 only (else null): 1/R, 1/m, 1/I and c_i of the
+                    // particle in each slot, the divisions done once per rebuild
 };
 
 // Per-particle data a policy's contact law reads beside the state records

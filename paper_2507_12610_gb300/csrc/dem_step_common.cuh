@@ -27,6 +27,32 @@ __device__ __forceinline__ void count_and_flag(Ctl* ctl, uint32_t npair, uint32_
   }
 }
 
+// x in single precision, chopped, by integer instructions alone: a conversion
+// instruction takes the FP64 pipe's 16 cycles a warp.  Magnitudes below 2^-126
+// become at most 2^-126, those of 2^128 and more (and non-finite ones) the largest
+// float.
+__device__ __forceinline__ float chop(double x) {
+  const int hi = __double2hiint(x);
+  const int mag = min(max((hi & 0x7fffffff) - 0x38000000, 0), 0x0fefffff);  // new bias
+  const uint32_t b = __funnelshift_l((uint32_t)__double2loint(x), (uint32_t)mag, 3);
+  return __uint_as_float(b | ((uint32_t)hi & 0x80000000u));
+}
+
+// Conservative overlap test of two particles (x, y, z, R) without double-precision
+// arithmetic (with scale > 1: of particles within scale S); the contact law takes
+// the exact one.  Chopping moves a coordinate by
+// less than 2^-23 of itself, so for a touching pair the offset's length is off by
+// less than 2^-23 (|a|_1 + |b|_1) <= 2^-23 (2 |a|_1 + 2 S) in the 1-norm; 3e-7 covers
+// that, 1e-6 of S the chopped radii and the roundings here, and 1e-36 squares that
+// are not normal numbers.
+__device__ __forceinline__ bool near_chopped(const D4& a, const D4& b, float scale = 1.000001f) {
+  const float ax = chop(a.x), ay = chop(a.y), az = chop(a.z);
+  const float dx = ax - chop(b.x), dy = ay - chop(b.y), dz = az - chop(b.z);
+  const float S = chop(a.w) + chop(b.w);
+  const float reach = S * scale + 3e-7f * ((fabsf(ax) + fabsf(ay)) + (fabsf(az) + S));
+  return dx * dx + dy * dy + dz * dz <= reach * reach + 1e-36f;
+}
+
 // Hamilton product (Sec. 2.3).
 template <typename T>
 __device__ __forceinline__ void qmul(const T a[4], const T b[4], T out[4]) {

@@ -207,10 +207,12 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
 
     // B: contact law for 32 queued contacts at a time, then ordered
     // per-particle sums (a queued pair found apart by the exact test
-    // contributes zero and keeps no history)
+    // contributes zero, or nothing where the policy has a closer test, and keeps
+    // no history)
     for (uint32_t i0 = 0; i0 < qn; i0 += 32) {
       const uint32_t i = i0 + lane;
       CT c6[6] = {CT(0), CT(0), CT(0), CT(0), CT(0), CT(0)};
+      bool counts = false;
       if (i < qn) {
         const uint32_t code = S.qcode[i];
         const uint32_t u = S.qslot[i];
@@ -223,13 +225,16 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
         const Rec Wt = W[w0 + tl], Wu = W[u];
         const typename Pol::Aux At = Pol::aux(lb, w0 + tl), Au = Pol::aux(lb, u);
         Hist h = H[e];
-        if (Pol::pair(p, t_is_i, t_is_i ? Pt : Pu, t_is_i ? Pu : Pt, t_is_i ? Vt : Vu,
+        counts = Pol::closer(t_is_i ? Pt : Pu, t_is_i ? Pu : Pt);
+        if (counts &&
+            Pol::pair(p, t_is_i, t_is_i ? Pt : Pu, t_is_i ? Pu : Pt, t_is_i ? Vt : Vu,
                       t_is_i ? Vu : Vt, t_is_i ? Wt : Wu, t_is_i ? Wu : Wt, t_is_i ? At : Au,
                       t_is_i ? Au : At, h, stamp_now, stamp_new, c6)) {
           H[e] = h;
           ++npair;
         }
       }
+      const unsigned counted = Pol::kCloser ? __ballot_sync(full, counts) : 0u;
 #pragma unroll
       for (int c = 0; c < 6; ++c) S.contrib[lane][c] = c6[c];
       __syncwarp();
@@ -249,7 +254,9 @@ k_step_warp(Ctl* ctl, Params p, StateBufs sb, Lists L, MeshDev mesh, double* for
         const uint32_t a = ra > i0 ? ra : i0;
         const uint32_t b = rb < i0 + 32 ? rb : i0 + 32;
         CT h = S.acc_h[pp][c], l = S.acc_l[pp][c];
-        for (uint32_t jj = a; jj < b; ++jj) Pol::Acc::add1(h, l, S.contrib[jj - i0][c]);
+        for (uint32_t jj = a; jj < b; ++jj)
+          if (!Pol::kCloser || (counted >> (jj - i0) & 1u))
+            Pol::Acc::add1(h, l, S.contrib[jj - i0][c]);
         S.acc_h[pp][c] = h;
         S.acc_l[pp][c] = l;
       }
