@@ -3,9 +3,9 @@
 // force/torque gather, and the semi-implicit Euler + SPIRAL integration
 // (arXiv 2507.12610, Sec. 2.1-2.3).
 //
-// One thread per particle slot.  A thread walks its list in ascending partner
-// caller index, then its triangle candidates in ascending triangle index, and
-// sums the contributions in exactly that order: the result is deterministic
+// A warp takes the entries and contacts of its particles together
+// (dem_step_warp.cuh) and sums each particle's contributions in ascending partner
+// caller index, then in ascending triangle index: the result is deterministic
 // and independent of the launch shape, the skin and the rebuild schedule (no
 // floating-point atomics anywhere).  Each touching pair is evaluated by both
 // of its particles in the canonical orientation (lower caller index = body i),

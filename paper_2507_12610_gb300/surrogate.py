@@ -11,10 +11,10 @@ bias is carried by a constant-1 input column):
                  M_i  = sum over neighbours j of m_ij (receiver i)
                  h_i += relu([h_i, M_i, 1] W_u)                    272 -> 128
   decoder        y_i = [h_i, 1] W_d   (6 outputs: a_i, R_i alpha_i) 144 -> 6
-The neighbour graph joins particles closer than 2.2 R_max.  Every matrix
-product, gather, segment sum, transpose, loss and Adam update runs in the
-kernels of mpnn.cu (include/mpnn.h); this module only allocates buffers
-(PyTorch device memory) and sequences the calls.  Sums follow the graph's
+The neighbour graph joins particles closer than 2.2 R_max.  The graph, the
+loss and the Adam update run in the kernels of mpnn.cu, the layers forward in
+mpnn_layers.cu and backward in mpnn_grad.cu (include/mpnn.h); this module only
+allocates buffers (PyTorch device memory) and sequences the calls.  Sums follow the graph's
 CSR order, so forward and backward passes are deterministic.
 """
 from __future__ import annotations
