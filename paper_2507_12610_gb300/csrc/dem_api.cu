@@ -281,7 +281,7 @@ inline void split(double a, float& hi, float& lo) {
 cudaError_t enqueue_step(dem_scene* s, cudaStream_t st) {
   const bool turning = !s->static_mesh;
   const bool inside = turning && step_poses(s->p);
-  launch_spawn(st, s->ctl, s->p, s->sb, s->bb, s->mesh);
+  launch_spawn(st, s->ctl, s->p, s->sb, s->L, s->bb, s->mesh);
   cudaError_t e = cudaSuccess;
   if (turning && !inside) {
     e = cudaEventRecord(s->pose_fork, st);
@@ -1180,7 +1180,7 @@ int dem_step_timed(dem_scene* s, int64_t nsteps, double* phase_ms) {
     if (!s->static_mesh) launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 1);
     cudaEventRecord(ev[1], s->stream);
     launch_rebuild(s->stream, s->ctl, s->p, s->sb, s->L, s->bb, s->mesh);
-    launch_spawn(s->stream, s->ctl, s->p, s->sb, s->bb, s->mesh);
+    launch_spawn(s->stream, s->ctl, s->p, s->sb, s->L, s->bb, s->mesh);
     cudaEventRecord(ev[2], s->stream);
     launch_step(s->stream, s->ctl, s->p, s->sb, s->L, s->mesh, s->forces, false);
     cudaEventRecord(ev[3], s->stream);

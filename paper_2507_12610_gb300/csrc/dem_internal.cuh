@@ -161,7 +161,9 @@ struct ListBuf {
   uint8_t* back;    // [offs[n]] for an entry whose partner has the higher caller index,
                     // the index of this particle in the partner's list
   D4* inv;          // [n] DEM_FP64 only (else null): 1/R, 1/m, 1/I and c_i of the
-                    // particle in each slot, the divisions done once per rebuild
+                    // particle in each slot, the divisions done once per rebuild (of
+                    // a spawned one by the spawn kernel: its first step is before the
+                    // next rebuild)
 };
 
 // Per-particle data a policy's contact law reads beside the state records
@@ -262,10 +264,23 @@ __device__ __forceinline__ ListBuf list_of(const Lists& L, uint32_t b) {
   r.inv = b ? L.b[1].inv : L.b[0].inv;
   return r;
 }
+
+// 1/R, 1/m, 1/I and the drag coefficient c_i of a DEM_FP64 particle, each
+// division written as the step's law and integrator write it, so with the same
+// bits; zero for a row awaiting spawning.  (Only DEM_FP64 keeps them.)
+__device__ __forceinline__ D4 inverses(const Params& p, const D4& P, const D4& V) {
+  const double R = P.w, mass = V.w;
+  if (R == 0.0) return make_D4(0.0, 0.0, 0.0, 0.0);
+  const double I = 2.0 / 5.0 * mass * R * R;
+  return make_D4(1.0 / R, 1.0 / mass, 1.0 / I, 9.0 * p.eta / (2.0 * p.rho * R * R));
+}
+__device__ __forceinline__ D4 inverses(const Params&, const F8&, const F8&) {
+  return make_D4(0.0, 0.0, 0.0, 0.0);
+}
 #endif
 
 // Kernel launch helpers implemented in the .cu files.
-void launch_spawn(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, BinBuf bb,
+void launch_spawn(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L, BinBuf bb,
                   MeshDev mesh);
 // The pose of step ctl->step + ahead (ahead 0 or 1) into the pose arrays.
 void launch_mesh_pose(cudaStream_t st, const Ctl* ctl, const Params& p, MeshDev mesh, int ahead);

@@ -46,19 +46,6 @@ __device__ __forceinline__ float4 posf_of(const Params& p, const void* state, ui
                      (float)(P.z - p.origin[2]), (float)P.w);
 }
 
-// 1/R, 1/m, 1/I and the drag coefficient c_i of a DEM_FP64 particle, each
-// division written as the step's law and integrator write it, so with the same
-// bits; zero for a row awaiting spawning.  (Only DEM_FP64 keeps them.)
-__device__ __forceinline__ D4 inverses(const Params& p, const D4& P, const D4& V) {
-  const double R = P.w, mass = V.w;
-  if (R == 0.0) return make_D4(0.0, 0.0, 0.0, 0.0);
-  const double I = 2.0 / 5.0 * mass * R * R;
-  return make_D4(1.0 / R, 1.0 / mass, 1.0 / I, 9.0 * p.eta / (2.0 * p.rho * R * R));
-}
-__device__ __forceinline__ D4 inverses(const Params&, const F8&, const F8&) {
-  return make_D4(0.0, 0.0, 0.0, 0.0);
-}
-
 // Vertex slot j of element k at the reference pose, shifted and rounded like
 // the pose arrays (unused slots repeat vertex 0); w = the vertex count in slot 0.
 __device__ __forceinline__ float4 ref_vertex(const Params& p, const MeshDev& mesh, int4 tv,

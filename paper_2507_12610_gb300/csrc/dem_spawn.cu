@@ -18,7 +18,8 @@
 // particles sit at the end of the slot order in caller order, see the binning),
 // and the control block asks for a list rebuild at the next step.  A new
 // particle cannot touch anything at the positions of this step, so it needs no
-// list entries before that rebuild.
+// list entries before that rebuild; what the step reads of it beside its state
+// (DEM_FP64: ListBuf::inv, whose c_i is the drag of that first step) is written here.
 //
 // Compiled without FMA contraction: the centre and radius of a kept sphere
 // are the same bits as those of the plain evaluation of the same formulas.
@@ -127,7 +128,7 @@ constexpr int kSpawnWarps = 16;
 
 template <typename Rec>
 __global__ void __launch_bounds__(32 * kSpawnWarps)
-k_spawn(Ctl* ctl, Params p, StateBufs sb, BinBuf bb, MeshDev mesh) {
+k_spawn(Ctl* ctl, Params p, StateBufs sb, Lists L, BinBuf bb, MeshDev mesh) {
   __shared__ double kx[kSpawnMaxAttempts], ky[kSpawnMaxAttempts], kz[kSpawnMaxAttempts],
       kr[kSpawnMaxAttempts];
   __shared__ uint32_t free_s[kSpawnWarps];  // the warp's attempt overlaps nothing
@@ -222,8 +223,11 @@ k_spawn(Ctl* ctl, Params p, StateBufs sb, BinBuf bb, MeshDev mesh) {
     const unsigned ok = __ballot_sync(full, lane < nb && free_s[lane < nb ? lane : 0] != 0u);
     const int first = __ffs((int)ok) - 1;  // -1: all failed
     if (first == wid && lane == 0) {
-      put_new(p, P, static_cast<Rec*>(buf_of(sb.V, ph)), static_cast<Rec*>(buf_of(sb.W, ph)),
-              static_cast<Rec*>(buf_of(sb.Q, ph)), A + kept, cx, cy, cz, r);
+      Rec* V = static_cast<Rec*>(buf_of(sb.V, ph));
+      put_new(p, P, V, static_cast<Rec*>(buf_of(sb.W, ph)), static_cast<Rec*>(buf_of(sb.Q, ph)),
+              A + kept, cx, cy, cz, r);
+      D4* inv = list_of(L, ctl->lphase & 1u).inv;
+      if (inv) inv[A + kept] = inverses(p, P[A + kept], V[A + kept]);
       kx[kept] = cx;
       ky[kept] = cy;
       kz[kept] = cz;
@@ -246,13 +250,13 @@ k_spawn(Ctl* ctl, Params p, StateBufs sb, BinBuf bb, MeshDev mesh) {
 
 }  // namespace
 
-void launch_spawn(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, BinBuf bb,
+void launch_spawn(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists L, BinBuf bb,
                   MeshDev mesh) {
   if (p.sp_attempts <= 0) return;
   if (p.mixed)
-    k_spawn<F8><<<1, 32 * kSpawnWarps, 0, st>>>(ctl, p, sb, bb, mesh);
+    k_spawn<F8><<<1, 32 * kSpawnWarps, 0, st>>>(ctl, p, sb, L, bb, mesh);
   else
-    k_spawn<D4><<<1, 32 * kSpawnWarps, 0, st>>>(ctl, p, sb, bb, mesh);
+    k_spawn<D4><<<1, 32 * kSpawnWarps, 0, st>>>(ctl, p, sb, L, bb, mesh);
 }
 
 }  // namespace dem
