@@ -648,7 +648,8 @@ def bench_surrogate(dem, strm, n=100_000):
     torch.cuda.synchronize()
     net_ms = (time.perf_counter() - t0) * 1e3 / k
     surrogate._mesh_kw.clear()
-    surrogate._mesh_kw.update(verts=d["verts"], tris=d["tris"], tri_radius=d["tri_radius"])
+    surrogate._mesh_kw.update(verts=d["verts"], tris=d["tris"], tri_radius=d["tri_radius"],
+                              max_mesh_contacts=d["max_mesh_contacts"])
     one = surrogate.rollout(model, st, d["R"], d["params"], 1, overlap_growth=1e9,
                             energy_limit=1e9)
     hyb = surrogate.rollout(model, st, d["R"], d["params"], 3)

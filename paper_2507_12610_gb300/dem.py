@@ -316,6 +316,7 @@ class Scene:
         kw.setdefault("spawn", s.get("spawn"))
         kw.setdefault("material", s.get("material"))
         kw.setdefault("material_mu", s.get("material_mu"))
+        kw.setdefault("max_mesh_contacts", s.get("max_mesh_contacts", 0))
         return cls(s["params"], s["R"], s["x"], s.get("v"), s.get("w"), s.get("q"),
                    s.get("verts"), s.get("tris"), s.get("tri_radius"), s.get("elems"),
                    s.get("elem_radius"), **kw)

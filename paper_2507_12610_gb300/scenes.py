@@ -253,6 +253,10 @@ def drum_scene(n=1_000_000, seed=5, n_theta=128, n_rings=15, r_range=(0.8e-3, 1.
 
     nn_dist is the lattice nearest-neighbour distance (default 2 R_max plus a
     small gap, i.e. no overlaps); a smaller value gives initial overlaps.
+
+    max_mesh_contacts is the element capacity a grain needs: the n_theta
+    triangles of an end cap meet at its hub, and a loose grain that rolls past
+    there has all of them in its list (elsewhere no more than the default 16).
     """
     rng = np.random.default_rng(seed)
     r0, r1 = r_range
@@ -286,6 +290,7 @@ def drum_scene(n=1_000_000, seed=5, n_theta=128, n_rings=15, r_range=(0.8e-3, 1.
     s = _scene("drum", seed, params, R, X, v, w, q, V, T, np.zeros(len(T)), (dlo, dhi))
     s["drum_radius"] = radius
     s["drum_length"] = length
+    s["max_mesh_contacts"] = min(max(n_theta, 16), 255)  # (255: the library's limit)
     return s
 
 

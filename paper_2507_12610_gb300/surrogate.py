@@ -484,7 +484,8 @@ def experiment(n_scenes=16, n_train=80, n_eval=16, iters=3000, lr=1e-3, drum_n=1
     dem_stride_ms = (time.perf_counter() - t0) * 1e3 / 10
     sc.close()
     _mesh_kw.clear()
-    _mesh_kw.update(verts=d["verts"], tris=d["tris"], tri_radius=d["tri_radius"])
+    _mesh_kw.update(verts=d["verts"], tris=d["tris"], tri_radius=d["tri_radius"],
+                    max_mesh_contacts=d["max_mesh_contacts"])
     roll = rollout(model, st, d["R"], d["params"], strides)
     # network time for one stride of the drum: graph + forward
     import torch
