@@ -12,8 +12,8 @@
 // test: the particles of the 27 cells around the centre (binned at the last list
 // rebuild; they have moved less than the skin since, and a cell is wider than
 // two radii plus the skin), the spheres kept earlier in the event, and the mesh
-// elements listed for the centre's cell; spheres and elements clearly apart in
-// single precision are left out of the double-precision test.  Kept particles
+// elements listed for the centre's cell; spheres clearly apart in single precision,
+// and elements whose box is, are left out of the double-precision test.  Kept particles
 // take the next inactive caller index, whose slot is its caller index (inactive
 // particles sit at the end of the slot order in caller order, see the binning),
 // and the control block asks for a list rebuild at the next step.  A new
@@ -124,6 +124,22 @@ __device__ __forceinline__ bool clearly_apart(const Params&, const float4&, cons
   return false;
 }
 
+// Whether point C is farther than reach from the box around an element's vertices
+// v[0 .. 3], in single precision.  No element is nearer than its box, and the box's
+// distance is off by the coordinates' rounding alone; a single-precision closest
+// point is off by more on thin triangles (0.4 mm on one of 16 mm x 10 um: the
+// sphere would be kept inside the wall).
+__device__ __forceinline__ bool outside_box(const float4& C, const float4* v, float reach) {
+  const float4 a = v[0], b = v[1], c = v[2], d = v[3];  // (unused slots repeat vertex 0)
+  const auto out = [](float x, float p, float q, float r, float s) {
+    const float lo = fminf(fminf(p, q), fminf(r, s)), hi = fmaxf(fmaxf(p, q), fmaxf(r, s));
+    return fmaxf(fmaxf(lo - x, x - hi), 0.f);
+  };
+  const float dx = out(C.x, a.x, b.x, c.x, d.x), dy = out(C.y, a.y, b.y, c.y, d.y),
+              dz = out(C.z, a.z, b.z, c.z, d.z);
+  return dx * dx + dy * dy + dz * dz > reach * reach;
+}
+
 constexpr int kSpawnWarps = 16;
 
 template <typename Rec>
@@ -200,16 +216,9 @@ k_spawn(Ctl* ctl, Params p, StateBufs sb, Lists L, BinBuf bb, MeshDev mesh) {
         for (uint32_t i = bb.tcell_start[cell] + lane; i < e && !ov; i += 32) {
           const uint32_t k = bb.tcell_tri[i];
           const uint32_t kp = pose + k;
-          const float4 Af = mesh.curf[4 * kp], Bf = mesh.curf[4 * kp + 1],
-                       Cf = mesh.curf[4 * kp + 2], Df = mesh.curf[4 * kp + 3];
-          const int nvk = (int)Af.w;
-          const V3<float> qf = mk(C.x, C.y, C.z);
-          const V3<float> yf =
-              closest_point_element(qf, mk(Af.x, Af.y, Af.z), mk(Bf.x, Bf.y, Bf.z),
-                                    mk(Cf.x, Cf.y, Cf.z), mk(Df.x, Df.y, Df.z), nvk);
-          const V3<float> df = qf - yf;
-          const float reach = C.w + (float)mesh.rad[k] + 4.f * p.mesh_prefilter;
-          if (dot(df, df) > reach * reach) continue;
+          const float4* vf = mesh.curf + 4 * (size_t)kp;
+          if (outside_box(C, vf, C.w + (float)mesh.rad[k] + 4.f * p.mesh_prefilter)) continue;
+          const int nvk = (int)vf[0].w;
           const V3<double> y = closest_point_element(
               mk(cx, cy, cz), xyz(mesh.cur[4 * kp]), xyz(mesh.cur[4 * kp + 1]),
               xyz(mesh.cur[4 * kp + 2]), xyz(mesh.cur[4 * kp + 3]), nvk);
