@@ -145,6 +145,15 @@ int mpnn_message_sums(int64_t n, int64_t E, const int64_t* off, const int32_t* n
                       const uint16_t* Wm, const float* p1, uint16_t* Mb, uint32_t* mask,
                       void* stream);
 
+/* The same, with the number of tries of each bounded wait (< 0: the library's,
+ * 2^18; 0: every wait runs out at once) and a report: *status (device, may be
+ * NULL) becomes DEM_ERR_TIMEOUT if a wait ran out and is left alone otherwise.
+ * (The next layer's relu takes a NaN in Mb for 0.) */
+int mpnn_message_sums_checked(int64_t n, int64_t E, const int64_t* off, const int32_t* nbr,
+                              const int32_t* dst, const uint16_t* hb, const uint16_t* eb,
+                              const uint16_t* Wm, const float* p1, uint16_t* Mb, uint32_t* mask,
+                              int32_t tries, int32_t* status, void* stream);
+
 /* Node update: h += relu([hb_in, Mb, 1] Wu) (rows past n: plus nothing), hb =
  * bf16(h) (may be hb_in), then out = p1 for the next round (W_next the message
  * layer [128][400], out [npad][128]) or, with decode nonzero, the outputs

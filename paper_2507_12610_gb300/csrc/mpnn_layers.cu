@@ -144,6 +144,8 @@ struct MessageArgs {
   const float* P1;     // [npad][128] h W_m over the receiver's columns
   uint16_t* Mb;        // [npad][128] rows 0 .. n-1 written
   uint32_t* mask;      // [E][4] or NULL: bit c of row e: message component c > 0
+  int tries;           // of a wait
+  int32_t* status;     // or NULL: DEM_ERR_TIMEOUT if a wait ran out
 };
 
 // One block an SM owns a range of nodes (of about the same cost for every block:
@@ -331,10 +333,11 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
     // ---- issuer
     if (lane == 0) {
       const uint32_t idesc = tc_idesc(128, 128);
-      for (int t = 0; t < ntile; ++t) {
+      int t = 0;
+      for (; t < ntile; ++t) {
         const int b = t & 1, d = t & 3;
-        if (!mbar_wait(bar(&S.full[b]), (t >> 1) & 1, failed)) break;
-        if (!mbar_wait(bar(&S.ready[d]), (t >> 2) & 1, failed)) break;
+        if (!mbar_wait(bar(&S.full[b]), (t >> 1) & 1, failed, a.tries)) break;
+        if (!mbar_wait(bar(&S.ready[d]), (t >> 2) & 1, failed, a.tries)) break;
         tc_fence_after();
         const uint32_t x = base + (uint32_t)b * kStBytes;
 #pragma unroll
@@ -346,6 +349,9 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
                desc_plain(base + kMsgXc, 2048u), idesc, true);
         tc_commit(bar(&S.mdone[d]));
       }
+      // a block that gave up has nobody who waited for the last products: they must
+      // not outlive the stages and TMEM
+      if (t > 0) mbar_drain(bar(&S.mdone[(t - 1) & 3]), ((t - 1) >> 2) & 1);
     }
     __syncwarp();
   } else if (warp >= kCopyWarp) {
@@ -360,7 +366,8 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
         mbar_arrive(bar(&S.full[b ^ 1]));
       }
       // the products of tile t - 2 have read the stage
-      const bool ok = t < 2 || mbar_wait(bar(&S.mdone[(t - 2) & 3]), ((t - 2) >> 2) & 1, failed);
+      const bool ok = t < 2 || mbar_wait(bar(&S.mdone[(t - 2) & 3]), ((t - 2) >> 2) & 1, failed,
+                                         a.tries);
       if (!__all_sync(0xffffffffu, ok)) break;
       const int64_t t0 = e_begin + (int64_t)t * kTileE;
       const int idx = next;
@@ -392,7 +399,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       Start st;
       st.load(a, R, run, c, lane);
       if (t + 1 < ntile) R.load(a.dst, t0 + kTileE + 64 * half, e_begin, e_end, lane);
-      const bool ok = t < 4 || mbar_wait(bar(&S.dfree[d]), ((t - 4) >> 2) & 1, failed);
+      const bool ok = t < 4 || mbar_wait(bar(&S.dfree[d]), ((t - 4) >> 2) & 1, failed, a.tries);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       st.fill(a, run, tmem + lanes + 128u * d + 64u * half, c);
@@ -434,7 +441,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       if (lane < 2) run[nrun + lane] = make_int2(m, -1);
       __syncwarp();
       if (t + kSumGroups < ntile) receivers(t0 + kSumGroups * kTileE);
-      const bool ok = mbar_wait(bar(&S.mdone[d]), (t >> 2) & 1, failed);
+      const bool ok = mbar_wait(bar(&S.mdone[d]), (t >> 2) & 1, failed, a.tries);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       const uint32_t acc = tmem + lanes + 128u * d;
@@ -485,7 +492,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
       float s = 0.f;
       if (t > 0) {
         const bool came = mbar_wait(bar(&S.carried[(t - 1) & (kCarry - 1)]),
-                                    ((t - 1) / kCarry) & 1, failed);
+                                    ((t - 1) / kCarry) & 1, failed, a.tries);
         if (!__all_sync(0xffffffffu, came)) break;
         s = S.carry[(t - 1) & (kCarry - 1)][c];
       }
@@ -508,6 +515,7 @@ __global__ void __launch_bounds__(kMsgThreads, 1) k_message(MessageArgs a) {
   tc_fence_before();
   __syncthreads();
   if (S.failed) {  // a wait ran out: no sums that look like results
+    if (tid == 0 && a.status) *a.status = DEM_ERR_TIMEOUT;
     for (int64_t k = tid; k < (int64_t)(i1 - i0) * kH; k += kMsgThreads)
       a.Mb[(int64_t)i0 * kH + k] = 0x7FC0u;
   }
@@ -720,10 +728,19 @@ int mpnn_message_sums(int64_t n, int64_t E, const int64_t* off, const int32_t* n
                       const int32_t* dst, const uint16_t* hb, const uint16_t* eb,
                       const uint16_t* Wm, const float* p1, uint16_t* Mb, uint32_t* mask,
                       void* stream) {
+  return mpnn_message_sums_checked(n, E, off, nbr, dst, hb, eb, Wm, p1, Mb, mask, -1, nullptr,
+                                   stream);
+}
+
+int mpnn_message_sums_checked(int64_t n, int64_t E, const int64_t* off, const int32_t* nbr,
+                              const int32_t* dst, const uint16_t* hb, const uint16_t* eb,
+                              const uint16_t* Wm, const float* p1, uint16_t* Mb, uint32_t* mask,
+                              int32_t tries, int32_t* status, void* stream) {
   if (n <= 0 || n > 0x7fffffff || E < 0 || !off || (E > 0 && (!nbr || !dst || !eb)) || !hb ||
       !Wm || !p1 || !Mb || !aligned16(hb, eb, Wm, p1, Mb, mask))
     return DEM_ERR_INVALID;
-  MessageArgs a{n, E, off, nbr, dst, hb, eb, Wm, p1, Mb, mask};
+  const MessageArgs a{n,  E,  off, nbr,  dst,  hb, eb,
+                      Wm, p1, Mb,  mask, tries < 0 ? kMbarTries : tries, status};
   auto* k = mask ? &k_message<true> : &k_message<false>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMsgBytes) !=
       cudaSuccess) {

@@ -16,24 +16,36 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.b32 %0, 1, 0, p;\n}"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return done != 0u;
+}
+
 // Waits for the phase of the given parity, a bounded number of tries (a try
 // itself waits for a while): false if it did not come, or if another thread gave
 // up (*failed).  A thread that gives up says so in *failed.
 constexpr int kMbarTries = 1 << 18;
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* failed) {
-  for (int i = 0; i < kMbarTries; ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.b32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* failed,
+                                          int tries) {
+  for (int i = 0; i < tries; ++i) {
+    if (mbar_try(bar, parity)) return true;
     if (*failed) return false;
   }
   *failed = 1;
   return false;
+}
+
+// Waits for the phase whether or not another thread gave up: for the end of
+// operations that must not outlive what they read and write.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < kMbarTries && !mbar_try(bar, parity); ++i) {
+  }
 }
 
 __device__ __forceinline__ void fence_async_smem() {

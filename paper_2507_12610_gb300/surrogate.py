@@ -31,8 +31,9 @@ EXPORTS = ("mpnn_gemm", "mpnn_gemm_split", "mpnn_transpose_bf16", "mpnn_to_bf16"
            "mpnn_concat_rows", "mpnn_residual", "mpnn_gather_rows", "mpnn_segment_sum",
            "mpnn_segment_sum_cols", "mpnn_segment_sum_perm", "mpnn_relu_backward",
            "mpnn_adam", "mpnn_mse", "mpnn_encode_nodes", "mpnn_encode_edges",
-           "mpnn_message_sums", "mpnn_update_nodes", "mpnn_grad_decode", "mpnn_grad_update",
-           "mpnn_grad_messages", "mpnn_grad_nodes", "mpnn_grad_weights")
+           "mpnn_message_sums", "mpnn_message_sums_checked", "mpnn_update_nodes",
+           "mpnn_grad_decode", "mpnn_grad_update", "mpnn_grad_messages", "mpnn_grad_nodes",
+           "mpnn_grad_weights")
 
 H = 128          # hidden width
 ROUNDS = 3       # message-passing rounds
