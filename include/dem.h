@@ -44,9 +44,9 @@ extern "C" {
 #define DEM_ERR_INVALID 1   /* argument violates the requirements of Table 2 or the layout */
 #define DEM_ERR_CAPACITY 2  /* a neighbour or mesh-contact list overflowed its capacity */
 #define DEM_ERR_NONFINITE 3 /* a particle state became NaN or infinite */
-#define DEM_ERR_TIMEOUT 4   /* reserved for a bounded device wait that gives up; no
-                               kernel of this library waits on another (kernel
-                               boundaries order the phases), so none returns it */
+#define DEM_ERR_TIMEOUT 4   /* a bounded device wait gave up (the message kernel of
+                               mpnn.h, between the warps of a block; no kernel
+                               waits on another) */
 #define DEM_ERR_CUDA 5      /* a CUDA runtime call failed */
 #define DEM_ERR_NOMEM 6     /* device memory allocation failed */
 

@@ -131,6 +131,11 @@ int mpnn_relu_backward(int64_t n, const float* Y, float* G, void* stream);
 int mpnn_encode_nodes(int64_t n, int64_t npad, const uint16_t* nf, const uint16_t* Wn,
                       const uint16_t* Wm_next, float* h, uint16_t* hb, float* p1, void* stream);
 
+/* The same, and *status (device, may be NULL) = DEM_OK. */
+int mpnn_encode_nodes_checked(int64_t n, int64_t npad, const uint16_t* nf, const uint16_t* Wn,
+                              const uint16_t* Wm_next, float* h, uint16_t* hb, float* p1,
+                              int32_t* status, void* stream);
+
 /* Edge states: eb [E][128] = bf16(relu(ef We)) (ef [E][16]). */
 int mpnn_encode_edges(int64_t E, const uint16_t* ef, const uint16_t* We, uint16_t* eb,
                       void* stream);
@@ -148,7 +153,7 @@ int mpnn_message_sums(int64_t n, int64_t E, const int64_t* off, const int32_t* n
 /* The same, with the number of tries of each bounded wait (< 0: the library's,
  * 2^18; 0: every wait runs out at once) and a report: *status (device, may be
  * NULL) becomes DEM_ERR_TIMEOUT if a wait ran out and is left alone otherwise.
- * (The next layer's relu takes a NaN in Mb for 0.) */
+ * (The next layer's relu takes a NaN in Mb for 0: the status is what tells.) */
 int mpnn_message_sums_checked(int64_t n, int64_t E, const int64_t* off, const int32_t* nbr,
                               const int32_t* dst, const uint16_t* hb, const uint16_t* eb,
                               const uint16_t* Wm, const float* p1, uint16_t* Mb, uint32_t* mask,
@@ -162,6 +167,13 @@ int mpnn_message_sums_checked(int64_t n, int64_t E, const int64_t* off, const in
 int mpnn_update_nodes(int64_t n, int64_t npad, const uint16_t* hb_in, const uint16_t* Mb,
                       const uint16_t* Wu, const uint16_t* W_next, int32_t decode, float* h,
                       uint16_t* hb, float* out, uint32_t* mask, void* stream);
+
+/* The same; with decode, the outputs are NaN if *status (device, may be NULL) is
+ * not DEM_OK. */
+int mpnn_update_nodes_checked(int64_t n, int64_t npad, const uint16_t* hb_in, const uint16_t* Mb,
+                              const uint16_t* Wu, const uint16_t* W_next, int32_t decode,
+                              float* h, uint16_t* hb, float* out, uint32_t* mask,
+                              const int32_t* status, void* stream);
 
 /* Backward of the fused layers.  zb is the bf16 gradient of a layer's output
  * before its relu (zero where the relu cut it off); W the bf16 copies

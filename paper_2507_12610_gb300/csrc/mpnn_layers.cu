@@ -541,6 +541,7 @@ struct NodeArgs {
   uint16_t* hb;           // [npad][128]
   float* out;             // P1 [npad][128] or y [npad][64]
   uint32_t* mask;         // [npad][4] or NULL: bit c: update component c > 0
+  int32_t* status;        // or NULL; encode: cleared; decode: NaN outputs if it is set
 };
 
 constexpr int kTileN = 64;
@@ -564,6 +565,8 @@ __global__ void __launch_bounds__(kNodeGroups * kGroupThreads, 1) k_node(NodeArg
   const int lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3;
   const int wm = warp >> 2, wn = warp & 3;
+  if (Encode && a.status && blockIdx.x == 0 && threadIdx.x == 0) *a.status = DEM_OK;
+  const bool failed = Decode && a.status && *a.status != DEM_OK;
   const uint32_t base = smem_addr(smem_any);  // the weights
   uint8_t* const smem = smem_any + kNodeTiles + grp * kNodeTile;  // the group's tile
   const uint32_t tile = smem_addr(smem);
@@ -670,8 +673,9 @@ __global__ void __launch_bounds__(kNodeGroups * kGroupThreads, 1) k_node(NodeArg
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const int row = wm * 32 + 16 * i + 8 * h + g, c = wn * 32 + 8 * j + 2 * t4;
-            *reinterpret_cast<float2*>(a.out + (r0 + row) * kOut + c) =
-                make_float2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+            float2 v = make_float2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+            if (Decode && failed) v = make_float2(NAN, NAN);
+            *reinterpret_cast<float2*>(a.out + (r0 + row) * kOut + c) = v;
           }
     }
   }
@@ -697,6 +701,12 @@ extern "C" {
 
 int mpnn_encode_nodes(int64_t n, int64_t npad, const uint16_t* nf, const uint16_t* Wn,
                       const uint16_t* Wm_next, float* h, uint16_t* hb, float* p1, void* stream) {
+  return mpnn_encode_nodes_checked(n, npad, nf, Wn, Wm_next, h, hb, p1, nullptr, stream);
+}
+
+int mpnn_encode_nodes_checked(int64_t n, int64_t npad, const uint16_t* nf, const uint16_t* Wn,
+                              const uint16_t* Wm_next, float* h, uint16_t* hb, float* p1,
+                              int32_t* status, void* stream) {
   if (n <= 0 || npad < n || npad % kTileN || !nf || !Wn || !Wm_next || !h || !hb || !p1 ||
       !aligned16(nf, Wn, Wm_next, h, hb, p1))
     return DEM_ERR_INVALID;
@@ -709,6 +719,7 @@ int mpnn_encode_nodes(int64_t n, int64_t npad, const uint16_t* nf, const uint16_
   a.h = h;
   a.hb = hb;
   a.out = p1;
+  a.status = status;
   return launch_node<true, false>(a, static_cast<cudaStream_t>(stream));
 }
 
@@ -755,6 +766,14 @@ int mpnn_message_sums_checked(int64_t n, int64_t E, const int64_t* off, const in
 int mpnn_update_nodes(int64_t n, int64_t npad, const uint16_t* hb_in, const uint16_t* Mb,
                       const uint16_t* Wu, const uint16_t* W_next, int32_t decode, float* h,
                       uint16_t* hb, float* out, uint32_t* mask, void* stream) {
+  return mpnn_update_nodes_checked(n, npad, hb_in, Mb, Wu, W_next, decode, h, hb, out, mask,
+                                   nullptr, stream);
+}
+
+int mpnn_update_nodes_checked(int64_t n, int64_t npad, const uint16_t* hb_in, const uint16_t* Mb,
+                              const uint16_t* Wu, const uint16_t* W_next, int32_t decode,
+                              float* h, uint16_t* hb, float* out, uint32_t* mask,
+                              const int32_t* status, void* stream) {
   if (n <= 0 || npad < n || npad % kTileN || !hb_in || !Mb || !Wu || !W_next || !h || !hb ||
       !out || !aligned16(hb_in, Mb, Wu, W_next, h, hb, out, mask))
     return DEM_ERR_INVALID;
@@ -769,6 +788,7 @@ int mpnn_update_nodes(int64_t n, int64_t npad, const uint16_t* hb_in, const uint
   a.hb = hb;
   a.out = out;
   a.mask = mask;
+  a.status = const_cast<int32_t*>(status);  // (read only)
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   return decode ? launch_node<false, true>(a, st) : launch_node<false, false>(a, st);
 }

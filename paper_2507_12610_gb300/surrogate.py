@@ -30,8 +30,9 @@ EXPORTS = ("mpnn_gemm", "mpnn_gemm_split", "mpnn_transpose_bf16", "mpnn_to_bf16"
            "mpnn_graph", "mpnn_graph_cells", "mpnn_reverse_edges", "mpnn_features", "mpnn_gather_edges",
            "mpnn_concat_rows", "mpnn_residual", "mpnn_gather_rows", "mpnn_segment_sum",
            "mpnn_segment_sum_cols", "mpnn_segment_sum_perm", "mpnn_relu_backward",
-           "mpnn_adam", "mpnn_mse", "mpnn_encode_nodes", "mpnn_encode_edges",
-           "mpnn_message_sums", "mpnn_message_sums_checked", "mpnn_update_nodes",
+           "mpnn_adam", "mpnn_mse", "mpnn_encode_nodes",
+           "mpnn_encode_nodes_checked", "mpnn_encode_edges", "mpnn_message_sums",
+           "mpnn_message_sums_checked", "mpnn_update_nodes", "mpnn_update_nodes_checked",
            "mpnn_grad_decode", "mpnn_grad_update", "mpnn_grad_messages", "mpnn_grad_nodes",
            "mpnn_grad_weights")
 
@@ -153,6 +154,9 @@ class Graph:
 class MPNN:
     """The network's parameters (fp32 masters, bf16 copies, Adam moments)."""
 
+    # tries of a wait of the message kernel before it gives up (-1: the library's)
+    TRIES = -1
+
     def __init__(self, seed=0, weights=None):
         import torch
         self.torch = torch
@@ -198,7 +202,8 @@ class MPNN:
     # ---- forward -------------------------------------------------------------
     def forward(self, g: Graph, keep=True):
         """The outputs [npad][64] (fp32); keep: also the states and relu masks that
-        backward() needs."""
+        backward() needs.  Does not wait for the device; should a bounded wait in the
+        message kernel run out, all outputs are NaN and check() raises."""
         torch = self.torch
         f32, b16, i32 = torch.float32, torch.int16, torch.int32
         n, npad, E = g.n, g.npad, g.E
@@ -211,8 +216,11 @@ class MPNN:
         p1, y = new(npad, H, f32), new(npad, 64, f32)
         Mb, eb = new(npad, H, b16), new(g.Epad, H, b16)
         st = dict(hb=[hb], Mb=[], m=[], u=[], eb=eb)
+        self.report = new(1, 2, f32)  # the loss; the status of this pass
+        status = ctypes.c_void_p(self.report.data_ptr() + 4)
         _call("mpnn_encode_edges", E, g.ef, self.Wt["edge"], eb, None)
-        _call("mpnn_encode_nodes", n, npad, g.nf, self.Wt["node"], self.Wt["msg0"], h, hb, p1, None)
+        _call("mpnn_encode_nodes_checked", n, npad, g.nf, self.Wt["node"], self.Wt["msg0"], h, hb,
+              p1, status, None)
         m = u = None
         for r in range(ROUNDS):
             last = r == ROUNDS - 1
@@ -222,14 +230,23 @@ class MPNN:
                 m, u = new(g.Epad, H // 32, i32), new(npad, H // 32, i32)
                 for key, t in (("hb", hb), ("Mb", Mb), ("m", m), ("u", u)):
                     st[key].append(t)
-            _call("mpnn_message_sums", n, E, g.off, g.nbr, g.dst, hb_in, eb, self.Wt[f"msg{r}"],
-                  p1, Mb, m, None)
-            _call("mpnn_update_nodes", n, npad, hb_in, Mb, self.Wt[f"upd{r}"],
+            _call("mpnn_message_sums_checked", n, E, g.off, g.nbr, g.dst, hb_in, eb,
+                  self.Wt[f"msg{r}"], p1, Mb, m, _i32(self.TRIES), status, None)
+            _call("mpnn_update_nodes_checked", n, npad, hb_in, Mb, self.Wt[f"upd{r}"],
                   self.Wt["dec" if last else f"msg{r + 1}"], _i32(last), h, hb,
-                  y if last else p1, u, None)
+                  y if last else p1, u, status, None)
         if keep:
             self.state = st
         return y
+
+    def check(self):
+        """Waits for the last forward pass and raises DemError if it did not run to
+        its end; returns the loss, if one was taken."""
+        loss, status = self.report.cpu().numpy().reshape(2, 1)
+        rc = int(status.view(np.int32)[0])
+        if rc != 0:
+            raise _dem.DemError(rc, "forward")
+        return float(loss[0])
 
     # ---- backward ------------------------------------------------------------
     def backward(self, g: Graph, dy):
@@ -273,14 +290,11 @@ class MPNN:
     def loss_and_grad(self, g: Graph, target):
         """MSE over the n x 6 outputs; target fp32 [npad][64] (zeros past 6
         columns and n rows).  Fills G and returns the loss."""
-        torch = self.torch
-        dev = torch.device("cuda")
         y = self.forward(g)
-        dy = torch.empty_like(y)
-        out = torch.zeros(1, dtype=torch.float32, device=dev)
-        _call("mpnn_mse", y.numel(), y, target, 1.0 / (g.n * OUT), dy, out, None)
+        dy = self.torch.empty_like(y)
+        _call("mpnn_mse", y.numel(), y, target, 1.0 / (g.n * OUT), dy, self.report, None)
         self.backward(g, dy)
-        return float(out.item()) / (g.n * OUT)
+        return self.check() / (g.n * OUT)
 
     def adam(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.t += 1
@@ -355,8 +369,10 @@ def train(model: MPNN, pairs, R, dt, stride=10, iters=300, lr=1e-3, log_every=50
 
 def predict(model: MPNN, state, R):
     g = make_graph(state["x"], state["v"], state["w"], R, float(R.max()))
-    y = model.forward(g, keep=False)
-    return y[:g.n, :OUT].cpu().numpy().astype(np.float64) * SCALES["a_s"]
+    y = model.forward(g, keep=False)[:g.n, :OUT].cpu().numpy()
+    if not np.isfinite(y).all():
+        model.check()
+    return y.astype(np.float64) * SCALES["a_s"]
 
 
 def evaluate(model: MPNN, pairs, R, dt, g_vec, stride=10):

@@ -45,3 +45,34 @@ def test_a_wait_that_runs_out_is_reported(sg, degrees, keep):  # noqa: F811
         assert torch.equal(Mb[~rows], ref[~rows])
         again, Mb = message_sums(sg, model, g, -1, keep)
         assert again == 0 and torch.equal(Mb, ref)
+
+
+def test_a_pass_whose_wait_ran_out_is_no_result(sg, monkeypatch):  # noqa: F811
+    import torch
+    rng = np.random.default_rng(7)
+    n = 3000
+    x = rng.uniform(0, 1.6e-3 * n ** (1 / 3), size=(n, 3))
+    state = dict(x=x, v=rng.normal(scale=0.1, size=(n, 3)), w=rng.normal(size=(n, 3)))
+    R = np.full(n, 1e-3)
+    g = sg.make_graph(state["x"], state["v"], state["w"], R, 1e-3)
+    model = sg.MPNN(seed=3)
+    T = sg.target_buffer(rng.normal(size=(n, sg.OUT)), g.npad)
+    y = model.forward(g, keep=False)
+    loss = model.loss_and_grad(g, T)
+    G = {k: v.clone() for k, v in model.G.items()}
+
+    monkeypatch.setattr(sg.MPNN, "TRIES", 0)
+    for keep in (False, True):
+        assert bool(torch.isnan(model.forward(g, keep=keep)[:n, :sg.OUT]).all())
+        with pytest.raises(sg._dem.DemError, match="timed out"):
+            model.check()
+    with pytest.raises(sg._dem.DemError, match="timed out"):
+        model.loss_and_grad(g, T)
+    with pytest.raises(sg._dem.DemError, match="timed out"):
+        sg.predict(model, state, R)
+
+    monkeypatch.setattr(sg.MPNN, "TRIES", -1)
+    assert torch.equal(model.forward(g, keep=False), y)
+    assert model.loss_and_grad(g, T) == loss
+    assert all(torch.equal(model.G[k], v) for k, v in G.items())
+    assert np.isfinite(sg.predict(model, state, R)).all()
