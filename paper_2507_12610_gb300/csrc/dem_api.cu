@@ -25,6 +25,15 @@ namespace {
 // step 11.1 us, batches of 1 / 4 / 8 / 16 steps 10.2 / 4.5 / 3.4 / 2.9 us.
 constexpr int kGraphSteps = 8;
 
+// A captured batch of steps: as the body of a loop over batches, so that one launch
+// runs all the steps asked for, or (where the driver refuses conditional nodes) as it
+// is, one batch a launch.
+struct StepGraph {
+  int steps;
+  cudaGraphExec_t exec = nullptr;
+  bool loop = false;
+};
+
 // Device memory of a scene: cudaMalloc, or the caller's allocator
 // (dem_scene_create_with_allocator).  Every block is released with the scene.
 struct Alloc {
@@ -175,15 +184,12 @@ struct dem_scene {
   double* forces = nullptr;
   double* export_buf = nullptr;  // [13 n] state read-back staging (caller order)
   Alloc mem;
-  // step graphs with 1 and kGraphSteps steps per batch (conditional graphs: a
-  // loop over batches, so one launch runs any number of steps; else one batch)
-  cudaGraphExec_t exec1 = nullptr, execG = nullptr;
+  StepGraph step1{1}, stepG{kGraphSteps};
   cudaStream_t aux = nullptr;  // captures the bodies of the loop node
   // captures the rebuild bodies, and the branch of a step that computes the
   // next step's mesh pose beside the step kernels (fork and join events)
   cudaStream_t pose_stream = nullptr;
   cudaEvent_t pose_fork = nullptr, pose_join = nullptr;
-  bool conditional_graphs = false;
   bool static_mesh = true;
 };
 
@@ -370,35 +376,38 @@ cudaError_t enqueue_loop(dem_scene* s, int nsteps) {
   return e != cudaSuccess ? e : e2;
 }
 
-// The graph of nsteps steps a batch.
-int build_graph(dem_scene* s, int nsteps, cudaGraphExec_t* out) {
+// Captures the step graph if it is not there yet.
+int build_graph(dem_scene* s, StepGraph& sg) {
+  if (sg.exec) return DEM_OK;
   // first choice: conditional nodes; fall back to the plain sequence (rebuild
   // kernels that return at once) if the driver refuses.
   // DEM_GRAPH_CONDITIONAL=0 in the environment keeps every rebuild kernel a
-  // plain graph node (profilers cannot see kernels of conditional graphs)
+  // plain graph node (profilers cannot see kernels of conditional graphs), 8
+  // those of the one-step graph alone
   const char* env = std::getenv("DEM_GRAPH_CONDITIONAL");
-  const bool allow_cond = !(env && env[0] == '0');
+  const bool allow_cond = !(env && (env[0] == '0' || (env[0] == '8' && sg.steps == 1)));
   for (int attempt = 0; attempt < 2; ++attempt) {
     const bool cond = attempt == 0 && s->aux != nullptr && allow_cond;
     cudaGraph_t g = nullptr;
     DEM_TRY(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     if (cond) {
-      e = enqueue_loop(s, nsteps);
+      e = enqueue_loop(s, sg.steps);
     } else {
-      for (int i = 0; i < nsteps && e == cudaSuccess; ++i) {
+      for (int i = 0; i < sg.steps && e == cudaSuccess; ++i) {
         launch_rebuild(s->stream, s->ctl, s->p, s->sb, s->L, s->bb, s->mesh);
         e = enqueue_step(s, s->stream);
       }
     }
     const cudaError_t e2 = cudaStreamEndCapture(s->stream, &g);
     if (e == cudaSuccess && e2 == cudaSuccess) {
-      e = cudaGraphInstantiate(out, g, 0);
+      e = cudaGraphInstantiate(&sg.exec, g, 0);
       cudaGraphDestroy(g);
       if (e == cudaSuccess) {
-        s->conditional_graphs = cond;
+        sg.loop = cond;
         return DEM_OK;
       }
+      sg.exec = nullptr;
     } else if (g) {
       cudaGraphDestroy(g);
     }
@@ -679,8 +688,8 @@ int upload_state(dem_scene* s, const double* x, const double* v, const double* w
 
 void destroy(dem_scene* s) {
   if (!s) return;
-  if (s->exec1) cudaGraphExecDestroy(s->exec1);
-  if (s->execG) cudaGraphExecDestroy(s->execG);
+  if (s->step1.exec) cudaGraphExecDestroy(s->step1.exec);
+  if (s->stepG.exec) cudaGraphExecDestroy(s->stepG.exec);
   if (s->stream) cudaStreamSynchronize(s->stream);
   s->mem.release();
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
@@ -1126,8 +1135,8 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
   // capture and instantiate the step graphs now, so that no dem_step call
   // pays for it on the host while the device waits; a failure here leaves
   // them to be built on first use
-  if (build_graph(s, 1, &s->exec1) != DEM_OK) s->exec1 = nullptr;
-  if (build_graph(s, kGraphSteps, &s->execG) != DEM_OK) s->execG = nullptr;
+  build_graph(s, s->step1);
+  build_graph(s, s->stepG);
   cudaGetLastError();
   *out = s;
   return DEM_OK;
@@ -1136,29 +1145,23 @@ int dem_scene_create_with_allocator(const dem_params* params, const dem_particle
 int dem_step(dem_scene* s, int64_t nsteps) {
   if (!s || nsteps < 0) return DEM_ERR_INVALID;
   if (nsteps == 0) return DEM_OK;
-  // graphs are built on first use if creation could not; the first build says
-  // whether they loop on the device
-  const auto ready = [s](int k) {
-    cudaGraphExec_t* ex = k == 1 ? &s->exec1 : &s->execG;
-    return *ex ? (int)DEM_OK : build_graph(s, k, ex);
-  };
-  // a batch's steps beyond those left return at once (~1 us each); so do the
-  // loop's nodes (~8 us a batch): batches of one step pay for one or two steps
-  const int k = nsteps > 2 ? kGraphSteps : 1;
-  int rc = ready(k);
-  if (rc != DEM_OK) return rc;
+  // graphs are built on first use if creation could not
   launch_set_left(s->stream, s->ctl, nsteps);
   DEM_TRY(cudaGetLastError());
-  if (s->conditional_graphs) {
-    DEM_TRY(cudaGraphLaunch(k == 1 ? s->exec1 : s->execG, s->stream));
-    return DEM_OK;
-  }
   for (int64_t left = nsteps; left > 0;) {
-    const int m = left >= kGraphSteps ? kGraphSteps : 1;
-    rc = ready(m);
+    // a batch's steps beyond those left return at once (~1 us each); so do the
+    // loop's nodes (~8 us a batch): batches of one step pay for one or two steps
+    StepGraph* sg = left > 2 ? &s->stepG : &s->step1;
+    int rc = build_graph(s, *sg);
     if (rc != DEM_OK) return rc;
-    DEM_TRY(cudaGraphLaunch(m == 1 ? s->exec1 : s->execG, s->stream));
-    left -= m;
+    if (!sg->loop) {  // whole batches only
+      sg = left >= kGraphSteps ? &s->stepG : &s->step1;
+      rc = build_graph(s, *sg);
+      if (rc != DEM_OK) return rc;
+    }
+    DEM_TRY(cudaGraphLaunch(sg->exec, s->stream));
+    if (sg->loop) return DEM_OK;
+    left -= sg->steps;
   }
   return DEM_OK;
 }
@@ -1295,7 +1298,7 @@ int dem_get_stats(dem_scene* s, dem_stats* out) {
   const int32_t rebuild_launches = 9 + (s->p.pair_res ? 1 : 0);
   const int32_t base = (s->static_mesh || step_poses(s->p) ? 0 : 1) + 2 +
                        (s->p.sp_attempts > 0 ? 1 : 0) + (s->p.pair_res ? 1 : 0);
-  if (s->conditional_graphs) {
+  if ((s->stepG.exec ? s->stepG : s->step1).loop) {
     out->launches_per_step = base;
     out->launches_per_rebuild = rebuild_launches;
   } else {
