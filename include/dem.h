@@ -112,9 +112,11 @@ typedef struct dem_params {
   int32_t spawn_every;      /* steps between spawn events; <= 0 selects 1 */
   uint64_t spawn_seed;
   int32_t step_warps;       /* warps per block of the contact/integration kernel:
-                               4 or 8; <= 0 selects 4 (a tuning knob for scenes of
-                               more than 80,000 particles, results do not depend
-                               on it) */
+                               4 or 8; <= 0 selects 4.  A tuning knob, results do not
+                               depend on it; it has an effect with more than 81,920
+                               rows (max(n, n_max)) in DEM_MIXED, 40,960 in
+                               DEM_MIXED64, and none in DEM_FP64 (but with
+                               DEM_FP64_TWO_SIDED=1, as DEM_MIXED64) */
   int32_t reserved;
 } dem_params;
 

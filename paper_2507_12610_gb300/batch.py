@@ -194,15 +194,21 @@ def discharged(batch, x):
 def autotune(batch, precision=1, skins=None, block_warps=(4, 8), steps=200, warmup=50,
              dem=None):
     """Pick the list skin and the step kernel's warps per block by timing
-    short runs of the batch itself (device time per step, CUDA events around
-    whole graph replays).  Returns (best, table)."""
+    short runs of the batch itself (wall time per step).  Returns (best, table);
+    where the block shape selects no other kernel, a skin's one run stands for
+    all its rows."""
+    from . import dem as rules
     if dem is None:
-        from . import dem
+        dem = rules
     rmax = float(np.max(batch["R"]))
     skins = skins or [0.1 * rmax, 0.2 * rmax, 0.35 * rmax, 0.5 * rmax]
+    matters = rules.step_warps_matters(len(batch["R"]), precision)
     table = []
     for sk in skins:
-        for bw in block_warps:
+        for k, bw in enumerate(block_warps):
+            if k > 0 and not matters and bw in (4, 8):
+                table.append(dict(table[-1], step_warps=bw))
+                continue
             sc = dem.Scene.from_dict(batch, precision=precision, skin=sk, step_warps=bw)
             sc.step(warmup)
             sc.synchronize()

@@ -190,6 +190,16 @@ def contact_forces_noalloc(params: dict, n: int, r_max: float, R_ptr: int, x_ptr
                                               x_ptr, v_ptr, w_ptr, F_ptr, T_ptr, st))
 
 
+def step_warps_matters(rows: int, precision: int) -> bool:
+    """Whether step_warps selects between kernels for a scene of this many rows:
+    smaller ones run with fewer particles a warp and 4 warps a block
+    (particles_per_warp in csrc/dem_step_warp.cuh), DEM_FP64 with kernels of its
+    own block shape unless DEM_FP64_TWO_SIDED=1."""
+    if precision == DEM_FP64 and not os.environ.get("DEM_FP64_TWO_SIDED", "").startswith("1"):
+        return False
+    return rows > (81920 if precision == DEM_MIXED else 40960)
+
+
 def probe_fp64_fma(iters: int = 16384, stream=None) -> float:
     """FP64 FMA throughput of the current device (FMAs per second)."""
     lib = load()
