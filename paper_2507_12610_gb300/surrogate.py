@@ -101,8 +101,9 @@ def _upload(arrays, dev):
     host = torch.empty(start[-1], dtype=torch.float32)
     for a, k in zip(arrays, start):
         part = host[k:k + a.size].view(a.shape)
-        if a.dtype in (np.float64, np.float32) and a.flags.writeable and a.dtype.isnative \
-                and min(a.strides, default=0) >= 0:
+        # what torch converts (by its threads); numpy takes the rest
+        if a.dtype in (np.float64, np.float32) and a.dtype.isnative and a.flags.writeable \
+                and a.flags.aligned and all(st >= 0 and st % a.itemsize == 0 for st in a.strides):
             part.copy_(torch.from_numpy(a))
         else:
             part.numpy()[...] = a
