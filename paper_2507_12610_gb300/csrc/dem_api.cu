@@ -417,6 +417,12 @@ int build_graph(dem_scene* s, StepGraph& sg) {
   return DEM_ERR_CUDA;
 }
 
+// Host data goes to the device by copies on the default stream, which s->stream need
+// not follow, and a copy of a small pageable buffer may return before it has landed.
+// Called after the last copy, before kernels that read the data (the element cell
+// lists are built right after an upload, and only if the control block says so).
+int uploads_landed() { return cuda_status(cudaStreamSynchronize(nullptr)); }
+
 int read_ctl(dem_scene* s, Ctl* c) {
   DEM_TRY(cudaStreamSynchronize(s->stream));
   DEM_TRY(cudaMemcpy(c, s->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
@@ -671,10 +677,8 @@ int upload_state(dem_scene* s, const double* x, const double* v, const double* w
     DEM_TRY(cudaMemset(s->L.b[b].meta, 0, n * 4));
     DEM_TRY(cudaMemset(s->L.b[b].offs, 0, (n + 1) * 4));
   }
-  {
-    const int rc = clear_histories(s);
-    if (rc != DEM_OK) return rc;
-  }
+  int rc = clear_histories(s);
+  if (rc != DEM_OK) return rc;
   Ctl c{};
   c.step = step;
   c.rebuild = 1;
@@ -682,6 +686,8 @@ int upload_state(dem_scene* s, const double* x, const double* v, const double* w
   c.spawn_carry = spawn_carry;
   c.spawn_draws = spawn_draws;
   DEM_TRY(cudaMemcpy(s->ctl, &c, sizeof c, cudaMemcpyHostToDevice));
+  rc = uploads_landed();
+  if (rc != DEM_OK) return rc;
   launch_set_pose(s->stream, s->ctl, s->p);  // rotation of this step, on the device
   return DEM_OK;
 }
@@ -1449,6 +1455,8 @@ int dem_load(dem_scene* s, const void* buf, size_t len) {
   c.spawn_draws = draws;
   c.spawn_carry = carry;
   DEM_TRY(cudaMemcpy(s->ctl, &c, sizeof c, cudaMemcpyHostToDevice));
+  rc = uploads_landed();
+  if (rc != DEM_OK) return rc;
   launch_set_pose(s->stream, s->ctl, s->p);
   launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 0);
   launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 1);
