@@ -686,10 +686,7 @@ int upload_state(dem_scene* s, const double* x, const double* v, const double* w
   c.spawn_carry = spawn_carry;
   c.spawn_draws = spawn_draws;
   DEM_TRY(cudaMemcpy(s->ctl, &c, sizeof c, cudaMemcpyHostToDevice));
-  rc = uploads_landed();
-  if (rc != DEM_OK) return rc;
-  launch_set_pose(s->stream, s->ctl, s->p);  // rotation of this step, on the device
-  return DEM_OK;
+  return uploads_landed();
 }
 
 void destroy(dem_scene* s) {
@@ -1457,7 +1454,6 @@ int dem_load(dem_scene* s, const void* buf, size_t len) {
   DEM_TRY(cudaMemcpy(s->ctl, &c, sizeof c, cudaMemcpyHostToDevice));
   rc = uploads_landed();
   if (rc != DEM_OK) return rc;
-  launch_set_pose(s->stream, s->ctl, s->p);
   launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 0);
   launch_mesh_pose(s->stream, s->ctl, s->p, s->mesh, 1);
   DEM_TRY(cudaStreamSynchronize(s->stream));

@@ -29,7 +29,7 @@ struct Ctl {
   int64_t left;         // steps of the current dem_step call still to run
   int64_t rebuilds;
   double mesh_angle_ref;  // mesh rotation angle at the last rebuild
-  double rot_c, rot_s;    // cos / sin of the mesh rotation angle of the current step
+  double rot_c, rot_s;    // cos / sin of the mesh rotation angle, of the list rebuild
   uint32_t pair_contacts;  // touching directed pair entries, this step (accumulating)
   uint32_t mesh_contacts;
   uint32_t pair_contacts_last;  // ... of the last completed step
@@ -196,7 +196,7 @@ struct BinBuf {
   uint32_t* key;        // [n] cell of each slot (current order)
   uint32_t* local;      // [n] arrival index within its cell
   uint32_t* cell_count; // [ncells + 1], zero between rebuilds (the scan clears it)
-  uint32_t* cell_start; // [ncells + 1]
+  uint32_t* cell_start; // [ncells + 2] (one cell more: rows awaiting spawning)
   uint32_t* order;      // [n] old slots by cell, in arrival order within a cell
   uint32_t* src;        // [n] old slot of each new slot
   uint32_t* block_sums; // scan partials
@@ -296,8 +296,6 @@ void launch_advance(cudaStream_t st, Ctl* ctl, const Params& p);
 // q[n][4] one after another in `out` (13 n doubles, device memory).
 void launch_export_state(cudaStream_t st, const Ctl* ctl, const Params& p, StateBufs sb,
                          Lists L, int64_t n, double* out);
-// Sets ctl->rot_c / rot_s for the step in the control block.
-void launch_set_pose(cudaStream_t st, Ctl* ctl, const Params& p);
 // Sets the number of steps to run.
 void launch_set_left(cudaStream_t st, Ctl* ctl, int64_t left);
 // Sets a graph condition (inside a captured graph): whether the lists must be

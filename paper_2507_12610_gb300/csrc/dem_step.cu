@@ -41,8 +41,6 @@ __device__ __noinline__ void pose_block(const Params& p, const MeshDev& mesh, in
   const int k = block * blockDim.x + threadIdx.x;
   const int sin_thread = blockDim.x > 32 ? 32 : 0;
   if ((int)threadIdx.x == 0 || (int)threadIdx.x == sin_thread) {
-    // the same expression, so the same bits, as k_set_pose, which keeps the
-    // one-thread step kernels free of FP64 transcendentals
     const double th = p.omega_norm * ((double)step * p.dt);
     if (threadIdx.x == 0) s_cs[0] = p.omega_norm > 0.0 ? cos(th) : 1.0;
     if ((int)threadIdx.x == sin_thread) s_cs[1] = p.omega_norm > 0.0 ? sin(th) : 0.0;
@@ -97,14 +95,6 @@ __global__ void __launch_bounds__(kPoseThreads)
 k_mesh_pose(const Ctl* ctl, Params p, MeshDev mesh, int ahead) {
   if (ctl->status) return;  // the same for every thread of the block
   pose_block(p, mesh, ctl->step + ahead, blockIdx.x);
-}
-
-// Rotation of the mesh at the control block's step (after a host upload); the
-// same expression k_advance uses, so a resumed run sees the same bits.
-__global__ void k_set_pose(Ctl* ctl, Params p) {
-  const double th = p.omega_norm * ((double)ctl->step * p.dt);
-  ctl->rot_c = cos(th);
-  ctl->rot_s = sin(th);
 }
 
 // ---- graph condition: run the rebuild body of this step or skip it ----------
@@ -464,8 +454,7 @@ struct MixedPolicy {
     return true;
   }
 
-  // Element contacts (unless the caller took them already: with_mesh false)
-  // and integration of particle slot t.
+  // Integration of particle slot t from the sums of its contacts.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
                                                 int t, const F8& Pt, const F8& Vt,
@@ -726,9 +715,9 @@ struct Mixed64Policy {
     return true;
   }
 
-  // Element contacts (unless taken already) and integration of slot t: the
-  // accelerations and the SPIRAL increment in FP32 (from FP32 forces), added
-  // to the FP64 velocity, spin and orientation; positions advance in FP64.
+  // Integration of slot t: the accelerations and the SPIRAL increment in FP32
+  // (from FP32 forces), added to the FP64 velocity, spin and orientation;
+  // positions advance in FP64.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
                                                 int t, const D4& Pt, const D4& Vt,
@@ -823,10 +812,6 @@ void launch_step(cudaStream_t st, Ctl* ctl, const Params& p, StateBufs sb, Lists
 // the two meet where a step takes about 80 us.
 bool step_poses(const Params& p) {
   return p.n <= 200000 && p.hist32;
-}
-
-void launch_set_pose(cudaStream_t st, Ctl* ctl, const Params& p) {
-  k_set_pose<<<1, 1, 0, st>>>(ctl, p);
 }
 
 void launch_set_left(cudaStream_t st, Ctl* ctl, int64_t left) {

@@ -2,9 +2,10 @@
 // precision (arXiv 2507.12610, Sec. 2.1-2.3).  This translation unit is
 // compiled without floating-point contraction (--fmad=false), so every product
 // and sum is rounded as written, as in a plain double-precision program; the
-// kernel is the precision reference of the library.  The structure is the one
-// described in dem_step.cu: one thread per particle slot, partners in
-// ascending caller index, canonical pair orientation, no atomics on floats.
+// kernels are the precision reference of the library: each pair evaluated once and
+// gathered (dem_step_pairs.cuh) or, with DEM_FP64_TWO_SIDED=1, from both sides as
+// in dem_step.cu (dem_step_warp.cuh); partners in ascending caller index,
+// canonical pair orientation, no atomics on floats.
 #include "dem_geom.cuh"
 #include "dem_internal.cuh"
 #include "dem_law.cuh"
@@ -198,8 +199,7 @@ struct Fp64Policy {
     return true;
   }
 
-  // Element contacts (unless the caller took them already: with_mesh false)
-  // and integration of particle slot t.
+  // Integration of particle slot t from the sums of its contacts.
   static __device__ __forceinline__ void finish(const Params& p, const StateBufs& sb,
                                                 uint32_t ph, const ListBuf& lb,
                                                 int t, const D4& Pt, const D4& Vt,

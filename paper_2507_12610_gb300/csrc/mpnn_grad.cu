@@ -10,30 +10,12 @@
 // bytes that the nodes sum and the edge state's gradient.
 #include <algorithm>
 
-#include "../../include/dem.h"
 #include "../../include/mpnn.h"
 #include "mpnn_mma.cuh"
 
 namespace {
 
 using namespace mpnn;
-
-constexpr int kH = 128;
-constexpr uint32_t kRowH = 272;   // bytes of a staged row of 128 bf16 (17 pieces)
-constexpr uint32_t kRow64 = 144;  // ... of 64 bf16 (9 pieces)
-constexpr uint32_t kRow16 = 48;   // ... of 16 bf16 (3 pieces)
-constexpr int kSms = 152;
-
-int launch_status() {
-  return cudaGetLastError() == cudaSuccess ? DEM_OK : DEM_ERR_CUDA;
-}
-
-template <typename... P>
-bool aligned16(const P*... p) {
-  uintptr_t bits = 0;
-  ((bits |= reinterpret_cast<uintptr_t>(p)), ...);
-  return (bits & 15u) == 0;
-}
 
 // eight bf16 with those kept whose bit in `bits` is set
 __device__ __forceinline__ uint4 masked(uint4 v, uint32_t bits) {
@@ -63,7 +45,7 @@ struct InputGradArgs {
 };
 
 constexpr int kTile = 64;
-constexpr int kGroups = 2, kGroupThreads = 256;
+constexpr int kGroups = 2;
 
 template <Kind K>
 struct InputGrad {
@@ -73,10 +55,6 @@ struct InputGrad {
   static constexpr uint32_t kTiles = kCols * 128 * kRow;  // the rows follow the weights
   static constexpr uint32_t kBytes = kTiles + kGroups * kTile * kRow;
 };
-
-__device__ __forceinline__ void group_sync(int group) {
-  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kGroupThreads) : "memory");
-}
 
 // dX = dZ W^T, 64 rows a tile, 8 warps of 32 x 32 over 128 inputs at a time; two
 // groups of 8 warps share the weights in shared memory and walk over tiles, each

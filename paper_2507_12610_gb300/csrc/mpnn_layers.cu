@@ -14,7 +14,6 @@
 // 311 TFLOP/s on this chip, a sixth of tcgen05, and would bound them.
 #include <algorithm>
 
-#include "../../include/dem.h"
 #include "../../include/mpnn.h"
 #include "mpnn_mma.cuh"
 #include "mpnn_tc.cuh"
@@ -23,23 +22,8 @@ namespace {
 
 using namespace mpnn;
 
-constexpr int kH = 128;
-constexpr uint32_t kRowH = 272;    // bytes of a staged row of 128 bf16 (17 pieces)
-constexpr uint32_t kRow16 = 48;    // ... of 16 bf16 (3 pieces)
-constexpr uint32_t kRowK = 560;    // ... of 272 bf16 (35 pieces)
+constexpr uint32_t kRowK = 560;    // bytes of a staged row of 272 bf16 (35 pieces)
 constexpr uint32_t kRowDec = 304;  // ... of 144 bf16 (19 pieces)
-constexpr int kSms = 152;
-
-int launch_status() {
-  return cudaGetLastError() == cudaSuccess ? DEM_OK : DEM_ERR_CUDA;
-}
-
-template <typename... P>
-bool aligned16(const P*... p) {
-  uintptr_t bits = 0;
-  ((bits |= reinterpret_cast<uintptr_t>(p)), ...);
-  return (bits & 15u) == 0;
-}
 
 // rows x cols bf16 (columns c0 .. c0 + cols of a row-major matrix of row
 // length ld) into shared memory, rows `row` bytes apart, by all threads
@@ -545,7 +529,7 @@ struct NodeArgs {
 };
 
 constexpr int kTileN = 64;
-constexpr int kNodeGroups = 2, kGroupThreads = 256;
+constexpr int kNodeGroups = 2;
 constexpr uint32_t kNodeW = 0, kNodeW2 = kNodeW + 128 * kRowK, kNodeTiles = kNodeW2 + 128 * kRowH;
 constexpr uint32_t kNodeH = 0, kNodeM = kNodeH + kTileN * kRowH, kNodeTile = kNodeM + kTileN * kRowH;
 constexpr uint32_t kNodeBytes = kNodeTiles + kNodeGroups * kNodeTile;
@@ -554,10 +538,6 @@ constexpr uint32_t kNodeBytes = kNodeTiles + kNodeGroups * kNodeTile;
 // weights in shared memory and walks over tiles, each group its own (their loads
 // and barriers fill each other's gaps: 100,000 nodes 77 us, 97 us with one group;
 // 230 MB, 34 us, is the floor).  A tile a block first: few tiles use all SMs.
-__device__ __forceinline__ void group_sync(int group) {
-  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kGroupThreads) : "memory");
-}
-
 template <bool Encode, bool Decode>
 __global__ void __launch_bounds__(kNodeGroups * kGroupThreads, 1) k_node(NodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem_any[];

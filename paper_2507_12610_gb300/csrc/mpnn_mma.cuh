@@ -12,7 +12,32 @@
 
 #include <cstdint>
 
+#include "../../include/dem.h"
+
 namespace mpnn {
+
+constexpr int kSms = 152;
+constexpr int kH = 128;            // the network's width
+constexpr uint32_t kRowH = 272;    // bytes of a staged row of 128 bf16 (17 pieces)
+constexpr uint32_t kRow64 = 144;   // ... of 64 bf16 (9 pieces)
+constexpr uint32_t kRow16 = 48;    // ... of 16 bf16 (3 pieces)
+
+inline int launch_status() {
+  return cudaGetLastError() == cudaSuccess ? DEM_OK : DEM_ERR_CUDA;
+}
+
+template <typename... P>
+bool aligned16(const P*... p) {
+  uintptr_t bits = 0;
+  ((bits |= reinterpret_cast<uintptr_t>(p)), ...);
+  return (bits & 15u) == 0;
+}
+
+// A barrier of one of a block's groups of warps.
+constexpr int kGroupThreads = 256;
+__device__ __forceinline__ void group_sync(int group) {
+  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kGroupThreads) : "memory");
+}
 
 __device__ __forceinline__ uint16_t to_bf16(float x) {
   const __nv_bfloat16 b = __float2bfloat16_rn(x);

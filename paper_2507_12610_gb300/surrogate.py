@@ -186,7 +186,6 @@ class MPNN:
             self.G[name] = torch.zeros_like(self.W[name])
             self._refresh(name)
         self.t = 0
-        self.zero_bias = torch.zeros(256, dtype=torch.float32, device=dev)
 
     def _refresh(self, name):
         # bf16 copies through a zero-rate Adam step would move the moments;
