@@ -21,6 +21,7 @@ from __future__ import annotations
 
 import ctypes
 import math
+import struct
 
 import numpy as np
 
@@ -67,7 +68,8 @@ def load():
 
 # C arguments by Python type (other types: C values as they are, or tensors)
 _CONVERT = {int: ctypes.c_int64, float: ctypes.c_float, bool: ctypes.c_int32,
-            type(None): lambda _: ctypes.c_void_p(0), ctypes.c_int32: lambda v: v}
+            type(None): lambda _: ctypes.c_void_p(0), ctypes.c_int32: lambda v: v,
+            ctypes.c_void_p: lambda v: v}
 
 
 def _convert(a):
@@ -186,6 +188,8 @@ class MPNN:
             self.G[name] = torch.zeros_like(self.W[name])
             self._refresh(name)
         self.t = 0
+        # the last pass: its loss (a float) and, in the high half, its status
+        self.report = torch.zeros(1, dtype=torch.int64, device=dev)
 
     def _refresh(self, name):
         # bf16 copies through a zero-rate Adam step would move the moments;
@@ -216,7 +220,6 @@ class MPNN:
         p1, y = new(npad, H, f32), new(npad, 64, f32)
         Mb, eb = new(npad, H, b16), new(g.Epad, H, b16)
         st = dict(hb=[hb], Mb=[], m=[], u=[], eb=eb)
-        self.report = new(1, 2, f32)  # the loss; the status of this pass
         status = ctypes.c_void_p(self.report.data_ptr() + 4)
         _call("mpnn_encode_edges", E, g.ef, self.Wt["edge"], eb, None)
         _call("mpnn_encode_nodes_checked", n, npad, g.nf, self.Wt["node"], self.Wt["msg0"], h, hb,
@@ -242,11 +245,10 @@ class MPNN:
     def check(self):
         """Waits for the last forward pass and raises DemError if it did not run to
         its end; returns the loss, if one was taken."""
-        loss, status = self.report.cpu().numpy().reshape(2, 1)
-        rc = int(status.view(np.int32)[0])
+        loss, rc = struct.unpack("<fi", struct.pack("<q", self.report.item()))
         if rc != 0:
             raise _dem.DemError(rc, "forward")
-        return float(loss[0])
+        return loss
 
     # ---- backward ------------------------------------------------------------
     def backward(self, g: Graph, dy):
